@@ -431,16 +431,28 @@ struct edpc_session {
   uint64_t steps_total = 0, steps_run = 0;
   bool finished = false;
 
-  // CUDA graphs: `chunk` consecutive steps (so each step's FDM update can run
-  // under the next step's first layers), instantiated twice with separate
-  // timing events and launched alternately; and a one-step graph for step
-  // counts that do not fill a chunk.
-  cudaGraph_t g_chunk = nullptr, g_one = nullptr;
-  cudaGraphExec_t x_chunk[2] = {}, x_one = nullptr;
+  // CUDA graphs. x_run holds run_steps consecutive steps and x_one a single
+  // step, for step counts that do not fill the former; neither records events.
+  // An event-record node between two kernels costs the programmatic edge
+  // between them: around the two FDM launches such nodes left gaps of 5, 15
+  // and 12 us in the 425 us step of the 64 MiB mix. So the timed graphs
+  // (x_chunk: `chunk` steps, instantiated twice with separate events and
+  // launched alternately; x_one_t: one step) are made when profiling is first
+  // turned on.
+  // run_steps: instantiating and destroying a graph takes time in proportion
+  // to its nodes (about 60 a step). 16 steps instead of 64, instantiated once
+  // instead of twice, took opening and closing a session of the 64 MiB mix's
+  // model from 26 to 6 ms. Schedules that keep an FDM update running under the
+  // next step's layers join it at a graph's end, so they keep `chunk` steps.
+  cudaGraph_t g_run = nullptr, g_one = nullptr, g_chunk = nullptr, g_one_t = nullptr;
+  cudaGraphExec_t x_run = nullptr, x_one = nullptr, x_chunk[2] = {}, x_one_t = nullptr;
+  static constexpr int kRunSteps = 16;
+  int run_steps = kRunSteps;
   int graph_kernels = 0;  // kernels per step
 
   // FDM kernel timing: event set k of chunk execution p is tev[p * chunk + k];
-  // the one-step graph (and eager steps) use the sets after those.
+  // the one-step graph (and eager steps) use the sets after those. Made when
+  // profiling is first turned on.
   bool profiling = false;
   static constexpr int kChunk = 64;
   static constexpr int kEvSets = 2 * kChunk + 1;
@@ -457,6 +469,7 @@ struct edpc_session {
   int setup_common(const edpc_cfg& c, uint64_t n_, void* stream, const StreamLayout* explicit_lay = nullptr,
                    const std::vector<GroupInfo>* groups = nullptr);
   int capture_graph();
+  int capture_timed();
   int capture(int nsteps, int set0, cudaGraph_t* g);
   int launch_steps(uint64_t n);
   int code_pending();
@@ -469,9 +482,10 @@ edpc_session::~edpc_session() {
   if (st_coder) cudaStreamSynchronize(st_coder);
   for (auto& x : x_chunk)
     if (x) cudaGraphExecDestroy(x);
-  if (x_one) cudaGraphExecDestroy(x_one);
-  if (g_chunk) cudaGraphDestroy(g_chunk);
-  if (g_one) cudaGraphDestroy(g_one);
+  for (auto& x : {x_one, x_run, x_one_t})
+    if (x) cudaGraphExecDestroy(x);
+  for (auto& g : {g_chunk, g_one, g_run, g_one_t})
+    if (g) cudaGraphDestroy(g);
   for (auto& e : ev_model)
     if (e) cudaEventDestroy(e);
   for (auto& e : ev_coder)
@@ -563,14 +577,16 @@ int edpc_session::setup_common(const edpc_cfg& c, uint64_t n_, void* stream, con
   return EDPC_OK;
 }
 
-// Captures `nsteps` model steps (timing event sets set0, set0 + 1, ...) into
-// one graph that ends with every stream joined (the last FDM update waited for).
+// Captures `nsteps` model steps into one graph that ends with every stream
+// joined (the last FDM update waited for). set0 >= 0: with timing event sets
+// set0, set0 + 1, ...; -1: without event records.
 int edpc_session::capture(int nsteps, int set0, cudaGraph_t* g) {
-  model.timing = true;
+  model.timing = set0 >= 0;
   EDPC_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   int r = EDPC_OK;
   for (int k = 0; k < nsteps && r == EDPC_OK; ++k) {
-    for (int q = 0; q < kEv; ++q) model.ev_fdm[q] = tev[set0 + k][q];
+    if (set0 >= 0)
+      for (int q = 0; q < kEv; ++q) model.ev_fdm[q] = tev[set0 + k][q];
     io.tick = k;  // graphs start at even steps
     r = model.step(io, st);
   }
@@ -589,8 +605,8 @@ int edpc_session::capture(int nsteps, int set0, cudaGraph_t* g) {
 int edpc_session::capture_graph() {
   has_adam_ev = model.side_fdm != nullptr;
   if (!use_graph || steps_total == 0) return EDPC_OK;
-  chunk = kChunk;
-  EDPC_TRY(capture(1, 2 * kChunk, &g_one));
+  run_steps = model.side_fdm ? kChunk : kRunSteps;
+  EDPC_TRY(capture(1, -1, &g_one));
   EDPC_CUDA(cudaGraphInstantiate(&x_one, g_one, 0));
   size_t nn = 0;
   EDPC_CUDA(cudaGraphGetNodes(g_one, nullptr, &nn));
@@ -602,25 +618,42 @@ int edpc_session::capture_graph() {
     EDPC_CUDA(cudaGraphNodeGetType(nd, &t));
     if (t == cudaGraphNodeTypeKernel) ++graph_kernels;
   }
-  if (steps_total < (uint64_t)kChunk) return EDPC_OK;
-  EDPC_TRY(capture(kChunk, 0, &g_chunk));
-  EDPC_CUDA(cudaGraphInstantiate(&x_chunk[0], g_chunk, 0));
-  EDPC_CUDA(cudaGraphInstantiate(&x_chunk[1], g_chunk, 0));
-  // the second instantiation records into event sets kChunk .. 2 kChunk - 1
-  nn = 0;
-  EDPC_CUDA(cudaGraphGetNodes(g_chunk, nullptr, &nn));
-  nodes.resize(nn);
-  EDPC_CUDA(cudaGraphGetNodes(g_chunk, nodes.data(), &nn));
-  for (auto nd : nodes) {
-    cudaGraphNodeType t;
-    EDPC_CUDA(cudaGraphNodeGetType(nd, &t));
-    if (t != cudaGraphNodeTypeEventRecord) continue;
-    cudaEvent_t e;
-    EDPC_CUDA(cudaGraphEventRecordNodeGetEvent(nd, &e));
-    for (int k = 0; k < kChunk; ++k)
-      for (int q = 0; q < kEv; ++q)
-        if (e == tev[k][q]) EDPC_CUDA(cudaGraphExecEventRecordNodeSetEvent(x_chunk[1], nd, tev[kChunk + k][q]));
+  if (steps_total < (uint64_t)run_steps) return EDPC_OK;
+  EDPC_TRY(capture(run_steps, -1, &g_run));
+  EDPC_CUDA(cudaGraphInstantiate(&x_run, g_run, 0));
+  return EDPC_OK;
+}
+
+// The events and the graphs that profiling uses.
+int edpc_session::capture_timed() {
+  for (auto& set : tev)
+    for (auto& e : set)
+      if (!e) EDPC_CUDA(cudaEventCreate(&e));
+  if (!use_graph || steps_total == 0 || x_one_t) return EDPC_OK;
+  EDPC_CUDA(cudaStreamSynchronize(st));
+  EDPC_TRY(model.flush(st));  // an eager step's FDM update is waited for outside the capture
+  if (!g_one_t) EDPC_TRY(capture(1, 2 * kChunk, &g_one_t));
+  if (steps_total >= (uint64_t)kChunk) {
+    if (!g_chunk) EDPC_TRY(capture(kChunk, 0, &g_chunk));
+    for (auto& x : x_chunk)
+      if (!x) EDPC_CUDA(cudaGraphInstantiate(&x, g_chunk, 0));
+    // the second instantiation records into event sets kChunk .. 2 kChunk - 1
+    size_t nn = 0;
+    EDPC_CUDA(cudaGraphGetNodes(g_chunk, nullptr, &nn));
+    std::vector<cudaGraphNode_t> nodes(nn);
+    EDPC_CUDA(cudaGraphGetNodes(g_chunk, nodes.data(), &nn));
+    for (auto nd : nodes) {
+      cudaGraphNodeType t;
+      EDPC_CUDA(cudaGraphNodeGetType(nd, &t));
+      if (t != cudaGraphNodeTypeEventRecord) continue;
+      cudaEvent_t e;
+      EDPC_CUDA(cudaGraphEventRecordNodeGetEvent(nd, &e));
+      for (int k = 0; k < kChunk; ++k)
+        for (int q = 0; q < kEv; ++q)
+          if (e == tev[k][q]) EDPC_CUDA(cudaGraphExecEventRecordNodeSetEvent(x_chunk[1], nd, tev[kChunk + k][q]));
+    }
   }
+  EDPC_CUDA(cudaGraphInstantiate(&x_one_t, g_one_t, 0));
   return EDPC_OK;
 }
 
@@ -642,28 +675,33 @@ int edpc_session::harvest(int k) {
   return EDPC_OK;
 }
 
-// Launches the next n model steps: whole chunks through the chunk graph when
-// aligned, else one step at a time (one-step graph, or eagerly).
+// Launches the next n model steps: whole multi-step graphs when aligned, else
+// one step at a time (one-step graph, or eagerly).
 int edpc_session::launch_steps(uint64_t n) {
   uint64_t k = 0;
+  auto fits = [&](uint64_t j, int len) {
+    return j % len == 0 && n - k >= (uint64_t)len && steps_total - j >= (uint64_t)len;
+  };
   while (k < n) {
     const uint64_t j = steps_run;
     if (encoder && pipeline && j % chunk == 0 && j >= (uint64_t)(2 * chunk))
       EDPC_CUDA(cudaStreamWaitEvent(st, ev_coder[(j / chunk) % 2], 0));
     uint64_t adv = 1;
-    if (x_chunk[0] && j % chunk == 0 && n - k >= (uint64_t)chunk && steps_total - j >= (uint64_t)chunk) {
+    if (profiling && x_chunk[0] && fits(j, chunk)) {
       const int p = (int)((j / chunk) % 2);
-      if (profiling)
-        for (int q = 0; q < chunk; ++q) EDPC_TRY(harvest(p * chunk + q));
+      for (int q = 0; q < chunk; ++q) EDPC_TRY(harvest(p * chunk + q));
       EDPC_TRY(model.flush(st));  // an eager step's FDM update may still run on its own stream
       EDPC_CUDA(cudaGraphLaunch(x_chunk[p], st));
-      if (profiling)
-        for (int q = 0; q < chunk; ++q) tev_live[p * chunk + q] = true;
+      for (int q = 0; q < chunk; ++q) tev_live[p * chunk + q] = true;
       adv = (uint64_t)chunk;
+    } else if (!profiling && x_run && fits(j, run_steps)) {
+      EDPC_TRY(model.flush(st));
+      EDPC_CUDA(cudaGraphLaunch(x_run, st));
+      adv = (uint64_t)run_steps;
     } else if (x_one && !model.delayed) {  // (the delayed update alternates parities: eager)
       const int set = 2 * kChunk;
       if (profiling) EDPC_TRY(harvest(set));
-      EDPC_CUDA(cudaGraphLaunch(x_one, st));
+      EDPC_CUDA(cudaGraphLaunch(profiling ? x_one_t : x_one, st));
       if (profiling) tev_live[set] = true;
     } else {
       const int set = (int)(j % (2 * kChunk));
@@ -713,12 +751,6 @@ int edpc_session::join() {
   return EDPC_OK;
 }
 
-static int session_prepare_events(edpc_session* s) {
-  for (int k = 0; k < edpc_session::kEvSets; ++k)
-    for (int q = 0; q < edpc_session::kEv; ++q) EDPC_CUDA(cudaEventCreate(&s->tev[k][q]));
-  return EDPC_OK;
-}
-
 // Opens an encoder over the concatenation of `nparts` buffers (host, or
 // device when data_on_device). A single device buffer is used in place.
 // lay: explicit stream layout (file sets), else the balanced split.
@@ -748,7 +780,6 @@ static int encoder_open_impl(const edpc_cfg* cfg, const uint8_t* const* parts, c
   int r = gp ? s->setup_common(*cfg, len, cuda_stream, &gp->lay, &gp->groups)
              : s->setup_common(*cfg, len, cuda_stream, lay);
   if (r != EDPC_OK) return bail(r);
-  if ((r = session_prepare_events(s)) != EDPC_OK) return bail(r);
   cudaStream_t st = s->st;
   s->variant = variant;
   s->arch_L = arch_L;
@@ -994,7 +1025,6 @@ static int decoder_open_impl(const edpc_cfg& cfg, uint64_t n, const StreamLayout
   }
   int r = gp ? s->setup_common(cfg, n, cuda_stream, &gp->lay, &gp->groups) : s->setup_common(cfg, n, cuda_stream, lay);
   if (r != EDPC_OK) return bail(r);
-  if ((r = session_prepare_events(s)) != EDPC_OK) return bail(r);
   cudaStream_t st = s->st;
   const int b = s->b;
   if ((int)row_len.size() != b) return bail(fail(EDPC_ECORRUPT, "stream table does not match the layout"));
@@ -1135,6 +1165,7 @@ extern "C" int edpc_session_profile(edpc_session* s, int on) {
     for (int k = 0; k < edpc_session::kEvSets; ++k) EDPC_TRY(s->harvest(k));
   }
   if (on && !s->profiling) {
+    EDPC_TRY(s->capture_timed());
     s->fwd_ms = s->bwd_ms = s->adam_ms = 0;
     s->samples = 0;
   }
