@@ -921,22 +921,141 @@ cudaError_t launch_fdm_adam(const FdmSplitArgs& a, cudaStream_t st, bool persist
 // ============================================================================================
 // Embedding backward: scatter-add of dh0 into E's rows, owner computes.
 // CTA (c, q) owns byte value c and chunk q of kEmbChunkPos consecutive
-// positions. Warp w of 8 takes a contiguous eighth of the chunk, read 128
-// positions at a time (one 32-bit word per lane, coalesced, four words
-// prefetched); ballots find the positions p with ctx[p] == c, which the warp
-// visits in increasing p: lane d adds dh0[p][d] (and d + 32 when D > 32),
-// eight rows' loads in flight at a time. The 8 warp sums are added in warp
-// order. With one chunk that is dE[c]; with several, each CTA writes its
-// partial and the last CTA of c to arrive adds the chunks' partials in chunk
-// order (a fence precedes the arrival counter), so the result does not depend
-// on timing. Position p = s*K + k has its D gradient values at dX[p*D ..).
+// positions; warp w of 8 sums a contiguous eighth of the chunk in increasing
+// position (emb_range_sum). The 8 warp sums are added in warp order. With one
+// chunk that is dE[c]; with several, each CTA writes its partial and the last
+// CTA of c to arrive adds the chunks' partials in chunk order (a fence
+// precedes the arrival counter), so the result does not depend on timing.
+// Position p = s*K + k has its D gradient values at dX[p*D ..).
 // ============================================================================================
+// Per-warp scratch of emb_range_sum: a ring of kEmbStages stages of 256 floats
+// and the list of matching positions (a 256-position block and a remainder
+// below 32).
+constexpr int kEmbStages = 4;
+struct __align__(16) EmbScratch {
+  float ring[kEmbStages][256];
+  int list[256 + 32];
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// One warp's sum of the rows dX[p*D ..) over the positions p in [p_lo, p_hi)
+// with ctx[p] == c, in increasing p: lane d gets dimension d in a0 and d + 32 in a1.
+// What bounds it is the latency of the rows' loads when a byte value is
+// frequent (smooth images, spaces): the one warp then walks thousands of rows,
+// and the adds must stay in order. So the matches of 256 positions at a time
+// go into a list (ballots and prefix counts; the next positions' words are
+// already in flight) and their rows through a ring of asynchronous copies,
+// 1 KB a stage (256 / D rows), three stages ahead of the adds. With eight rows
+// in flight in registers instead, the 64 MiB mix's step spent 59 us here on
+// images and text; the adds' order, and so the bits, are the same.
+template <int DT>
+__device__ __forceinline__ void emb_range_sum(const uint8_t* __restrict__ ctx, const float* __restrict__ dX, int Drt,
+                                              uint32_t c, int p_lo, int p_hi, EmbScratch& s, float& a0, float& a1) {
+  const int lane = threadIdx.x & 31;
+  const int D = DT > 0 ? DT : Drt;
+  const int R = 256 / D, C4 = D / 4, n4 = R * C4;  // rows and 16-byte pieces (at most 64) of a stage
+  const int r0 = lane / C4, q0 = (lane - r0 * C4) * 4;
+  const int r1 = (lane + 32) / C4, q1 = (lane + 32 - r1 * C4) * 4;
+  const bool al4 = (reinterpret_cast<uintptr_t>(ctx) & 3) == 0 && (p_lo & 3) == 0;
+  a0 = a1 = 0.f;
+  int pend = 0, issued = 0, consumed = 0;
+  auto issue = [&](int first, int n) {
+    float* st = s.ring[issued % kEmbStages];
+    if (r0 < n && lane < n4) cp_async16(st + r0 * D + q0, dX + (size_t)s.list[first + r0] * D + q0);
+    if (r1 < n && lane + 32 < n4) cp_async16(st + r1 * D + q1, dX + (size_t)s.list[first + r1] * D + q1);
+    cp_async_commit();
+    ++issued;
+  };
+  auto add = [&](int n) {
+    const float* st = s.ring[consumed % kEmbStages];
+#pragma unroll
+    for (int r = 0; r < (DT > 0 ? 256 / (DT > 0 ? DT : 1) : n); ++r) {
+      if (r >= n) break;
+      if (lane < D) a0 += st[r * D + lane];
+      if (lane + 32 < D) a1 += st[r * D + lane + 32];
+    }
+    ++consumed;
+  };
+  auto word = [&](int pw) -> uint32_t {  // positions pw..pw+3 (a non-matching byte past p_hi)
+    if (al4 && pw + 4 <= p_hi) return *reinterpret_cast<const uint32_t*>(ctx + pw);
+    uint32_t x = 0;
+    for (int u = 0; u < 4; ++u) x |= (uint32_t)(pw + u < p_hi ? ctx[pw + u] : (uint8_t)(c ^ 1u)) << (8 * u);
+    return x;
+  };
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t nx[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) nx[k] = word(p_lo + k * 128 + 4 * lane);
+  for (int pb = p_lo; pb < p_hi; pb += 256) {
+    const uint32_t xs[2] = {nx[0], nx[1]};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) nx[k] = word(pb + 256 + k * 128 + 4 * lane);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      uint32_t at = (uint32_t)pend;
+      bool hit[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        hit[u] = ((xs[k] >> (8 * u)) & 0xffu) == c;
+        const uint32_t m = __ballot_sync(0xffffffffu, hit[u]);
+        at += __popc(m & below);
+        pend += __popc(m);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (hit[u]) s.list[at++] = pb + k * 128 + 4 * lane + u;
+    }
+    __syncwarp();
+    int done = 0;
+    for (; pend - done >= R; done += R) {  // warp-uniform
+      if (issued - consumed == kEmbStages) {
+        cp_async_wait<kEmbStages - 1>();
+        __syncwarp();
+        add(R);
+        __syncwarp();
+      }
+      issue(done, R);
+    }
+    if (done) {
+      pend -= done;
+      const int v = lane < pend ? s.list[done + lane] : 0;
+      __syncwarp();
+      if (lane < pend) s.list[lane] = v;
+    }
+    __syncwarp();
+  }
+  while (issued > consumed) {
+    cp_async_wait<0>();
+    __syncwarp();
+    add(R);
+  }
+  if (pend) {
+    __syncwarp();
+    issue(0, pend);
+    cp_async_wait<0>();
+    __syncwarp();
+    add(pend);
+  }
+}
+
+template <int DT>
 __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __restrict__ ctx,
                                                               const float* __restrict__ dX, int P, int D,
                                                               float* __restrict__ dE, float* __restrict__ part,
                                                               unsigned* __restrict__ cnt) {
   pdl_wait();
   pdl_launch();
+  __shared__ EmbScratch scratch[8];
   __shared__ float wsum[8][64];
   __shared__ int is_last;
   const uint32_t c = blockIdx.x;
@@ -945,59 +1064,8 @@ __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __r
   const int c_lo = min(P, q * kEmbChunkPos), c_hi = min(P, c_lo + kEmbChunkPos);
   const int per = ((c_hi - c_lo + 8 * 128 - 1) / (8 * 128)) * 128;  // positions per warp, a multiple of 128
   const int p_lo = min(c_hi, c_lo + w * per), p_hi = min(c_hi, p_lo + per);
-  const bool al4 = (reinterpret_cast<uintptr_t>(ctx) & 3) == 0;
-  float a0 = 0.f, a1 = 0.f;  // dims lane and lane + 32
-  int pend[8];
-  int np = 0;
-  auto flush = [&]() {
-    float v0[8], v1[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      v0[k] = (k < np && lane < D) ? dX[(size_t)pend[k] * D + lane] : 0.f;
-      v1[k] = (k < np && lane + 32 < D) ? dX[(size_t)pend[k] * D + lane + 32] : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      if (k < np) {
-        a0 += v0[k];
-        a1 += v1[k];
-      }
-    }
-    np = 0;
-  };
-  auto word = [&](int pw) -> uint32_t {  // positions pw..pw+3 (a non-matching byte past p_hi)
-    if (al4 && pw + 4 <= p_hi) return *reinterpret_cast<const uint32_t*>(ctx + pw);
-    uint32_t x = 0;
-    for (int u = 0; u < 4; ++u) x |= (uint32_t)(pw + u < p_hi ? ctx[pw + u] : (uint8_t)(c ^ 1u)) << (8 * u);
-    return x;
-  };
-  for (int pb = p_lo; pb < p_hi; pb += 4 * 128) {
-    uint32_t xs[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) xs[k] = (pb + k * 128 < p_hi) ? word(pb + k * 128 + 4 * lane) : (c ^ 1u) * 0x01010101u;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int p0 = pb + k * 128;
-      uint32_t m[4], any = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        m[u] = __ballot_sync(0xffffffffu, ((xs[k] >> (8 * u)) & 0xffu) == c);
-        any |= m[u];
-      }
-      while (any) {  // warp-uniform: lanes l in increasing order, then their bytes u
-        const int l = __ffs(any) - 1;
-        any &= any - 1;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if ((m[u] >> l) & 1u) {
-            pend[np++] = p0 + 4 * l + u;
-            if (np == 8) flush();
-          }
-        }
-      }
-    }
-  }
-  flush();
+  float a0, a1;  // dims lane and lane + 32
+  emb_range_sum<DT>(ctx, dX, D, c, p_lo, p_hi, scratch[w], a0, a1);
   wsum[w][lane] = a0;
   wsum[w][lane + 32] = a1;
   __syncthreads();
@@ -1036,24 +1104,27 @@ cudaError_t launch_embed_bwd(const uint8_t* ctx, const float* dX, int b, int K, 
   if (D > 64) return cudaErrorInvalidValue;
   const int nq = embed_bwd_chunks(b, K);
   if (nq > 1 && (!part || !cnt)) return cudaErrorInvalidValue;
-  return launch_k(embed_bwd_owner_kernel, dim3(256, nq < 1 ? 1 : nq), dim3(256), 0, st, ctx, dX, b * K, D, dE, part,
-                  cnt);
+  const dim3 grid(256, nq < 1 ? 1 : nq);
+  switch (D) {  // the configurations' widths have their loops unrolled
+    case 8: return launch_k(embed_bwd_owner_kernel<8>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
+    case 16: return launch_k(embed_bwd_owner_kernel<16>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
+    default: return launch_k(embed_bwd_owner_kernel<0>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
+  }
 }
 
 // Grouped embedding adjoint: CTA (group g, pair of byte values); warps 4v to
 // 4v + 3 own byte value 2 cb + v, each one quarter of the group's context
-// positions (in blocks of 512). A warp walks its quarter in increasing order,
-// 512 positions at a time (four 32-bit words of 4 positions per lane, loaded
-// together), finds the value's positions by ballot and adds their gradient
-// rows (lane d: dimensions d and d + 32) in position order, eight rows'
-// loads in flight at a time; the four quarter sums are then added in order.
-// So each dE[g][c] is a fixed-order sum that depends on the group alone.
+// positions (in blocks of 512), summed in increasing position
+// (emb_range_sum); the four quarter sums are then added in order. So each
+// dE[g][c] is a fixed-order sum that depends on the group alone.
+template <int DT>
 __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __restrict__ ctx,
                                                                const float* __restrict__ dX, int K, int D,
                                                                float* __restrict__ dE,
                                                                const GroupInfo* __restrict__ gi, size_t gs) {
   pdl_wait();
   pdl_launch();
+  __shared__ EmbScratch scratch[8];
   __shared__ float part[8][64];
   const GroupInfo g = gi[blockIdx.x];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1063,59 +1134,8 @@ __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __
   const int g_lo = g.r0 * K, g_hi = (g.r0 + g.s) * K;
   const int per = ((g_hi - g_lo + 4 * 512 - 1) / (4 * 512)) * 512;  // a quarter, whole 512-position blocks
   const int p_lo = min(g_hi, g_lo + (w & 3) * per), p_hi = min(g_hi, p_lo + per);
-  float a0 = 0.f, a1 = 0.f;
-  int pend[8];
-  int np = 0;
-  auto flush = [&]() {
-    float v0[8], v1[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      v0[k] = (k < np && lane < D) ? dX[(size_t)pend[k] * D + lane] : 0.f;
-      v1[k] = (k < np && lane + 32 < D) ? dX[(size_t)pend[k] * D + lane + 32] : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      if (k < np) {
-        a0 += v0[k];
-        a1 += v1[k];
-      }
-    }
-    np = 0;
-  };
-  for (int pb = p_lo; pb < p_hi; pb += 4 * 128) {
-    uint32_t xs[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      // positions pw..pw+3 (p_lo is a multiple of 4; bytes at or past p_hi never match)
-      const int pw = pb + k * 128 + 4 * lane;
-      uint32_t x = pw < p_hi ? *reinterpret_cast<const uint32_t*>(ctx + pw) : (c ^ 1u) * 0x01010101u;
-      for (int u = 0; u < 4; ++u)
-        if (pw + u >= p_hi) x = (x & ~(0xFFu << (8 * u))) | ((c ^ 1u) & 0xFFu) << (8 * u);
-      xs[k] = x;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int p0 = pb + k * 128;
-      uint32_t m[4], any = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        m[u] = __ballot_sync(0xffffffffu, ((xs[k] >> (8 * u)) & 0xffu) == c);
-        any |= m[u];
-      }
-      while (any) {  // warp-uniform: lanes in increasing order, then their bytes
-        const int l = __ffs(any) - 1;
-        any &= any - 1;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if ((m[u] >> l) & 1u) {
-            pend[np++] = p0 + 4 * l + u;
-            if (np == 8) flush();
-          }
-        }
-      }
-    }
-  }
-  flush();
+  float a0, a1;
+  emb_range_sum<DT>(ctx, dX, D, c, p_lo, p_hi, scratch[w], a0, a1);
   part[w][lane] = a0;
   part[w][lane + 32] = a1;
   __syncthreads();
@@ -1131,7 +1151,12 @@ cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, 
                                     const GroupInfo* gi, int ngroups, size_t gs, cudaStream_t st) {
   if (D > 64 || ngroups < 1 || ngroups > 65535 || !gi || (reinterpret_cast<uintptr_t>(ctx) & 3))
     return cudaErrorInvalidValue;
-  return launch_k(embed_bwd_groups_kernel, dim3(ngroups, 128), dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
+  const dim3 grid(ngroups, 128);
+  switch (D) {
+    case 8: return launch_k(embed_bwd_groups_kernel<8>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
+    case 16: return launch_k(embed_bwd_groups_kernel<16>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
+    default: return launch_k(embed_bwd_groups_kernel<0>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
+  }
 }
 
 // ============================================================================================
