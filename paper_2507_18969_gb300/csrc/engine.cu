@@ -561,19 +561,19 @@ int Model::refresh_bf16_weights(cudaStream_t st) {
 int Model::linear_fwd(const float* X, int rows, int in, size_t w_off, size_t b_off, int out, const float* resid,
                       float* Yo, cudaStream_t st) {
   const int epi = resid ? EPI_BIAS_RESID : EPI_BIAS;
-  GemmF32 g{rows, out, in, X, in, true, P + w_off, in, true, Yo, out, epi, P + b_off, resid, out};
+  GemmF32 g{rows, out, in, X, in, true, P + w_off, in, true, Yo, out, epi, P + b_off, resid, out, true};
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }
 
 int Model::linear_dx(const float* dOut, int rows, int out, size_t w_off, int in, float* dX, cudaStream_t st) {
-  GemmF32 g{rows, in, out, dOut, out, true, P + w_off, in, false, dX, in, EPI_STORE, nullptr, nullptr, 0};
+  GemmF32 g{rows, in, out, dOut, out, true, P + w_off, in, false, dX, in, EPI_STORE, nullptr, nullptr, 0, true};
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }
 
 int Model::linear_dw(const float* dOut, int rows, int out, const float* X, int in, size_t w_off, cudaStream_t st) {
-  GemmF32 g{out, in, rows, dOut, out, false, X, in, false, G + w_off, in, EPI_STORE, nullptr, nullptr, 0};
+  GemmF32 g{out, in, rows, dOut, out, false, X, in, false, G + w_off, in, EPI_STORE, nullptr, nullptr, 0, false};
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }

@@ -2,82 +2,178 @@
 //
 // This is the "plain FP32" arithmetic of the model's Linear layers
 // (Eqs. 10, 13, 14, 16, the head, and their adjoints). Each output element
-// sums its K products in increasing k order, so results are deterministic.
-// Tile 64 x 64 x 16, 256 threads, 4 x 4 outputs per thread (rows ty + 16i,
-// columns tx + 16j), operands staged through shared memory in [k][m] / [k][n]
-// order with coalesced global loads for either operand layout.
+// sums its K products in increasing k order by fused multiply-adds, so results
+// are deterministic and the same for every tile.
+//
+// Operands arrive by 16-byte asynchronous copies in STAGES stages of BKT = 32
+// values of k, in the layout they have in memory: an operand whose k is
+// contiguous as [m][k] rows of BKT + 4 floats (the padding puts eight
+// consecutive rows on distinct banks), one whose m is contiguous as [k][m]
+// rows. Either way a thread's TM (or TN) values of four consecutive k are TM
+// (TN) 16-byte shared-memory loads, and four k are TM * TN * 4 FMAs.
 #include "kernels.cuh"
 #include "launch.cuh"
 
+#include <mutex>
+
 namespace edpc {
 
-template <bool AK, bool BK, int EPI>
-__global__ void __launch_bounds__(256) gemm_f32_kernel(GemmF32 g) {
-  constexpr int BM = 64, BN = 64, BKT = 16;
+namespace {
+
+constexpr int BKT = 32;
+
+__device__ __forceinline__ void cp16(float* dst, const float* src, int bytes) {  // bytes < 16: zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src), "r"(bytes)
+               : "memory");
+}
+
+// One operand of a tile: ROWS rows (m or n) by BKT values of k.
+//   KC: k contiguous in memory; thread values r = t + i * T (T threads along the side)
+//   else: the rows are contiguous; thread values come in runs of V = min(4, TR):
+//         r = (i / V) * V * T + t * V + i % V
+template <bool KC, int ROWS, int TR>
+struct Operand {
+  static constexpr int T = ROWS / TR;
+  static constexpr int V = TR < 4 ? TR : 4;
+  static constexpr int LD = KC ? BKT + 4 : ROWS;
+  static constexpr int FLOATS = KC ? ROWS * LD : BKT * LD;
+  static constexpr int PIECES = ROWS * BKT / 4;  // 16-byte pieces of a stage
+  static_assert(KC || ROWS % 4 == 0, "rows are copied four at a time");
+
+  static __device__ __forceinline__ int row(int t, int i) {
+    return KC ? t + i * T : (i / V) * (V * T) + t * V + i % V;
+  }
+  template <int NT>
+  static __device__ __forceinline__ void load(float* s, const float* __restrict__ X, int ld, int r0, int rows, int k0,
+                                              int K, int tid) {
+#pragma unroll
+    for (int p = 0; p < (PIECES + NT - 1) / NT; ++p) {
+      const int e = tid + p * NT;
+      if (PIECES % NT && e >= PIECES) break;
+      if (KC) {
+        const int r = e / (BKT / 4), k = (e % (BKT / 4)) * 4;
+        const int left = (r0 + r < rows) ? K - (k0 + k) : 0;
+        const int n = left >= 4 ? 16 : (left > 0 ? left * 4 : 0);
+        cp16(s + r * LD + k, n ? X + (size_t)(r0 + r) * ld + k0 + k : X, n);
+      } else {
+        const int k = e / (ROWS / 4), r = (e % (ROWS / 4)) * 4;
+        const int left = (k0 + k < K) ? rows - (r0 + r) : 0;
+        const int n = left >= 4 ? 16 : (left > 0 ? left * 4 : 0);
+        cp16(s + k * LD + r, n ? X + (size_t)(k0 + k) * ld + r0 + r : X, n);
+      }
+    }
+  }
+  // f[q][i] = value of row(t, i) at k + q
+  static __device__ __forceinline__ void frag(const float* s, int t, int k, float (&f)[4][TR]) {
+    if (KC) {
+#pragma unroll
+      for (int i = 0; i < TR; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(s + row(t, i) * LD + k);
+        f[0][i] = v.x;
+        f[1][i] = v.y;
+        f[2][i] = v.z;
+        f[3][i] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float* p = s + (k + q) * LD;
+        if (V == 4) {
+#pragma unroll
+          for (int i = 0; i < TR; i += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p + row(t, i));
+            f[q][i] = v.x;
+            f[q][i + (V > 1 ? 1 : 0)] = v.y;
+            f[q][i + (V > 2 ? 2 : 0)] = v.z;
+            f[q][i + (V > 3 ? 3 : 0)] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < TR; ++i) f[q][i] = p[row(t, i)];
+        }
+      }
+    }
+  }
+};
+
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK>
+struct Tile {
+  using A = Operand<AK, BM, TM>;
+  using B = Operand<BK, BN, TN>;
+  static constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
+  static constexpr int WX = TX < 8 ? TX : 8, WY = 32 / WX;  // threads of a warp along n and m
+  static_assert(NT % 32 == 0 && TX % WX == 0 && TY % WY == 0, "whole warps");
+  static constexpr int STAGE = A::FLOATS + B::FLOATS;
+  static constexpr size_t kSmem = (size_t)STAGES * STAGE * sizeof(float);
+};
+
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI>
+__global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm_f32_kernel(const GemmF32 g) {
+  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK>;
+  extern __shared__ __align__(16) float smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tx = (warp % (S::TX / S::WX)) * S::WX + lane % S::WX;
+  const int ty = (warp / (S::TX / S::WX)) * S::WY + lane / S::WX;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int nk = (g.K + BKT - 1) / BKT;
+  auto load_a = [&](int kb) {
+    S::A::template load<S::NT>(smem + (kb % STAGES) * S::STAGE, g.A, g.lda, m0, g.M, kb * BKT, g.K, tid);
+  };
+  auto load_b = [&](int kb) {
+    S::B::template load<S::NT>(smem + (kb % STAGES) * S::STAGE + S::A::FLOATS, g.B, g.ldb, n0, g.N, kb * BKT, g.K,
+                               tid);
+  };
+  // Weights (b_early) were written at least two launches earlier, so their
+  // first stages are fetched before the dependent-launch wait.
+  if (g.b_early)
+    for (int q = 0; q < STAGES - 1 && q < nk; ++q) load_b(q);
   pdl_wait();
   pdl_launch();
-  __shared__ float As[BKT][BM + 4];
-  __shared__ float Bs[BKT][BN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[4][4];
+  for (int q = 0; q < STAGES - 1; ++q) {
+    if (q < nk) {
+      if (!g.b_early) load_b(q);
+      load_a(q);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
 
-  for (int k0 = 0; k0 < g.K; k0 += BKT) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int e = tid + r * 256;
-      int m, k;
-      if (AK) {
-        m = e >> 4;
-        k = e & 15;
-      } else {
-        k = e >> 6;
-        m = e & 63;
-      }
-      const int gm = m0 + m, gk = k0 + k;
-      float v = 0.f;
-      if (gm < g.M && gk < g.K) v = AK ? g.A[(size_t)gm * g.lda + gk] : g.A[(size_t)gk * g.lda + gm];
-      As[k][m] = v;
-      int n;
-      if (BK) {
-        n = e >> 4;
-        k = e & 15;
-      } else {
-        k = e >> 6;
-        n = e & 63;
-      }
-      const int gn = n0 + n, gk2 = k0 + k;
-      float w = 0.f;
-      if (gn < g.N && gk2 < g.K) w = BK ? g.B[(size_t)gn * g.ldb + gk2] : g.B[(size_t)gk2 * g.ldb + gn];
-      Bs[k][n] = w;
+  for (int kb = 0; kb < nk; ++kb) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();  // stage kb has landed for every thread, and stage kb - 1 has been read
+    if (kb + STAGES - 1 < nk) {
+      load_b(kb + STAGES - 1);
+      load_a(kb + STAGES - 1);
     }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* sa = smem + (kb % STAGES) * S::STAGE;
+    const float* sb = sa + S::A::FLOATS;
 #pragma unroll
-    for (int kk = 0; kk < BKT; ++kk) {
-      float a[4], bb[4];
+    for (int k = 0; k < BKT; k += 4) {
+      float a[4][TM], b[4][TN];
+      S::A::frag(sa, ty, k, a);
+      S::B::frag(sb, tx, k, b);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * bb[j];
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[q][i], b[q][j], acc[i][j]);
     }
-    __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + S::A::row(ty, i);
     if (m >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
+    for (int j = 0; j < TN; ++j) {
+      const int n = n0 + S::B::row(tx, j);
       if (n >= g.N) continue;
       float v = acc[i][j];
       if (EPI >= EPI_BIAS) v += g.bias[n];
@@ -87,22 +183,56 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(GemmF32 g) {
   }
 }
 
-template <bool AK, bool BK>
-static cudaError_t dispatch_epi(const GemmF32& g, dim3 grid, cudaStream_t st) {
-  switch (g.epi) {
-    case EPI_STORE: return launch_k(gemm_f32_kernel<AK, BK, EPI_STORE>, grid, dim3(256), 0, st, g);
-    case EPI_BIAS: return launch_k(gemm_f32_kernel<AK, BK, EPI_BIAS>, grid, dim3(256), 0, st, g);
-    default: return launch_k(gemm_f32_kernel<AK, BK, EPI_BIAS_RESID>, grid, dim3(256), 0, st, g);
-  }
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI>
+cudaError_t launch_one(const GemmF32& g, cudaStream_t st) {
+  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK>;
+  auto k = gemm_f32_kernel<BM, BN, TM, TN, STAGES, AK, BK, EPI>;
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [&] {
+    attr = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+  });
+  if (attr != cudaSuccess) return attr;
+  return launch_k(k, dim3(div_up(g.N, BN), div_up(g.M, BM)), dim3(S::NT), S::kSmem, st, g);
 }
+
+template <int BM, int BN, int TM, int TN, int STAGES>
+cudaError_t launch_tile(const GemmF32& g, cudaStream_t st) {
+  // the layouts the model uses: forward (A, B k-contiguous, with bias), input
+  // gradient (A only) and weight gradient (neither)
+  if (g.a_kcont && g.b_kcont) {
+    if (g.epi == EPI_BIAS) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BIAS>(g, st);
+    if (g.epi == EPI_BIAS_RESID) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BIAS_RESID>(g, st);
+  }
+  if (g.epi != EPI_STORE || g.b_kcont) return cudaErrorInvalidValue;
+  if (g.a_kcont) return launch_one<BM, BN, TM, TN, STAGES, true, false, EPI_STORE>(g, st);
+  return launch_one<BM, BN, TM, TN, STAGES, false, false, EPI_STORE>(g, st);
+}
+
+bool vec16(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0; }
+
+}  // namespace
 
 cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid(div_up(g.N, 64), div_up(g.M, 64));
-  if (g.a_kcont && g.b_kcont) return dispatch_epi<true, true>(g, grid, st);
-  if (g.a_kcont && !g.b_kcont) return dispatch_epi<true, false>(g, grid, st);
-  if (!g.a_kcont && g.b_kcont) return dispatch_epi<false, true>(g, grid, st);
-  return dispatch_epi<false, false>(g, grid, st);
+  // every width is a multiple of 8 and every tensor 16-byte aligned (checked, for the 16-byte copies)
+  if (!vec16(g.A, g.lda) || !vec16(g.B, g.ldb)) return cudaErrorInvalidValue;
+  // Tile by the number of outputs: the largest that still gives the 152 SMs
+  // work. A tile's chain over K is what the small ones wait for, so they take
+  // more CTAs of fewer values each; the large ones are bound by the shared
+  // memory's 128 bytes a cycle (TM + TN values in for TM * TN FMAs). Times in
+  // us with the tiles on either side (and of the former 64 x 64 tile with
+  // synchronous 4-byte loads), forward layout, M x N x K:
+  //   64 x 512 x 512     8x8 5.1, 8x16 6.4 (32.9)      128 x 512 x 512   8x8 9.3, 8x16 7.1, 16x32 8.8 (33.0)
+  //   512 x 256 x 512    8x16 10.0, 16x32 9.8 (33.3)   512 x 512 x 512   16x32 16.1, 32x64 14.7 (33.6)
+  //   1024 x 512 x 512   32x64 20.1, 64x64 22.1 (33.7) 1024 x 1024 x 2048 (weight gradient) 32x64 127.8,
+  //   64x64 106.1 (189.7)
+  const long long outs = (long long)g.M * g.N;
+  if (outs >= 1 << 20) return launch_tile<64, 64, 8, 4, 3>(g, st);
+  if (outs >= 192 << 10) return launch_tile<32, 64, 4, 4, 4>(g, st);
+  if (outs >= 96 << 10) return launch_tile<16, 32, 4, 2, 6>(g, st);
+  if (outs >= 48 << 10) return launch_tile<8, 16, 2, 2, 8>(g, st);
+  return launch_tile<8, 8, 2, 1, 8>(g, st);
 }
 
 }  // namespace edpc

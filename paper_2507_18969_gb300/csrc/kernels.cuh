@@ -194,6 +194,7 @@ struct GemmF32 {
   int epi;
   const float* bias;
   const float* R; int ldr;
+  bool b_early;  // B was written at least two launches before (weights): fetched ahead of the PDL wait
 };
 cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st);
 
