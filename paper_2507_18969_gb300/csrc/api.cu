@@ -1634,44 +1634,22 @@ extern "C" int edpc_range_encode(const uint32_t* sym, uint32_t nsym, uint32_t st
                                  uint32_t* out_len, void* stream) {
   if (!sym || !out || !out_len || streams == 0) return fail(EDPC_EINVAL, "NULL argument or no streams");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  EncState* es = nullptr;
-  unsigned long long* off = nullptr;
-  uint32_t* caps = nullptr;
-  std::vector<unsigned long long> h_off(streams);
-  std::vector<uint32_t> h_cap(streams, cap);
-  for (uint32_t s = 0; s < streams; ++s) h_off[s] = (unsigned long long)s * cap;
-  int r = EDPC_OK;
-  if (cudaMalloc(&es, sizeof(EncState) * streams) != cudaSuccess || cudaMalloc(&off, 8 * (size_t)streams) != cudaSuccess ||
-      cudaMalloc(&caps, 4 * (size_t)streams) != cudaSuccess) {
-    r = fail(EDPC_ENOMEM, "coder state");
-  } else {
-    cudaMemcpyAsync(off, h_off.data(), 8 * (size_t)streams, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(caps, h_cap.data(), 4 * (size_t)streams, cudaMemcpyHostToDevice, st);
-    Split none{0, 0, 0};
-    cudaError_t e = launch_prefix_encode(es, nullptr, none, 0, (int)streams, out, off, caps, st);
-    if (e == cudaSuccess) e = launch_range_encode(es, sym, (int)nsym, 0, (int)nsym, (int)streams, out, off, caps, st);
-    if (e == cudaSuccess) e = launch_encode_flush(es, (int)streams, out, off, caps, out_len, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) r = fail(EDPC_ECUDA, std::string("range encode: ") + cudaGetErrorString(e));
-    if (r == EDPC_OK) {
-      std::vector<uint32_t> l(streams);
-      cudaMemcpy(l.data(), out_len, 4 * (size_t)streams, cudaMemcpyDeviceToHost);
-      bool over = false;
-      for (auto& v : l)
-        if (v == 0xFFFFFFFFu) {
-          v = cap;
-          over = true;
-        }
-      if (over) {
-        cudaMemcpy(out_len, l.data(), 4 * (size_t)streams, cudaMemcpyHostToDevice);
-        r = fail(EDPC_EINVAL, "a stream needs more than cap bytes");
-      }
+  cudaError_t e = launch_range_encode_whole(sym, (int)nsym, (int)streams, out, cap, out_len, st);
+  std::vector<uint32_t> l(streams);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(l.data(), out_len, 4 * (size_t)streams, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return fail(EDPC_ECUDA, std::string("range encode: ") + cudaGetErrorString(e));
+  bool over = false;
+  for (auto& v : l)
+    if (v == 0xFFFFFFFFu) {
+      v = cap;
+      over = true;
     }
-  }
-  cudaFree(es);
-  cudaFree(off);
-  cudaFree(caps);
-  return r;
+  if (!over) return EDPC_OK;
+  EDPC_CUDA(cudaMemcpyAsync(out_len, l.data(), 4 * (size_t)streams, cudaMemcpyHostToDevice, st));
+  EDPC_CUDA(cudaStreamSynchronize(st));
+  return fail(EDPC_EINVAL, "a stream needs more than cap bytes");
 }
 
 // ==========================================================================================

@@ -108,14 +108,17 @@ __host__ __device__ inline int group_active(const GroupInfo& g, long long i) {
 constexpr int kGroupAlign = 64;  // rows per group are padded to a multiple of this
 
 // Range coder states (one per stream), kept in device memory between launches.
+// pend: the last `npend` code bytes (an integer of that many bytes, and a carry
+// out of them as the bit above), held back so that a carry out of `low` is one
+// addition; `pos` bytes are in the window.
 struct EncState {
-  unsigned long long low;
+  unsigned long long pend;
+  uint32_t low;
   uint32_t range;
-  uint32_t cache;
-  uint32_t pending;
-  uint32_t started;
+  uint32_t npend;
   uint32_t pos;
   uint32_t err;
+  uint32_t pad;
 };
 struct DecState {
   uint32_t code;

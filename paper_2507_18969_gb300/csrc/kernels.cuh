@@ -171,6 +171,10 @@ cudaError_t launch_prefix_encode(EncState* es, const uint8_t* data, Split sp, in
 cudaError_t launch_range_encode(EncState* es, const uint32_t* ring, int ring_slots, int slot0,
                                 int nsteps, int b, uint8_t* out, const unsigned long long* out_off,
                                 const uint32_t* out_cap, cudaStream_t st);
+// Whole streams in one launch, each into its own window of cap bytes of `out`:
+// out_len[s] = the stream's length, or 0xFFFFFFFF when it does not fit.
+cudaError_t launch_range_encode_whole(const uint32_t* sym, int nsteps, int b, uint8_t* out, uint32_t cap,
+                                      uint32_t* out_len, cudaStream_t st);
 cudaError_t launch_encode_flush(EncState* es, int b, uint8_t* out, const unsigned long long* out_off,
                                 const uint32_t* out_cap, uint32_t* out_len, cudaStream_t st);
 cudaError_t launch_dec_init(DecState* ds, const uint8_t* bits, const unsigned long long* off,
