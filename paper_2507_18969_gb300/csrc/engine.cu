@@ -11,7 +11,8 @@
 //   adjoint is fused with the FDM's Adam update. Adam on the shared params.
 //
 // Two arithmetic paths share this sequence:
-//   FP32  SIMT GEMMs and separate element-wise kernels.
+//   FP32  SIMT GEMMs and separate element-wise kernels; weight gradients and
+//         column sums on the side stream as below.
 //   BF16  tcgen05 GEMMs whose epilogues fuse the MBRB element-wise ops and
 //         write the BF16 (and transposed BF16) operands of the next GEMMs; the
 //         weight-gradient GEMMs and column sums, which nothing on the step's
@@ -316,11 +317,14 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
       }
     }
     if (!bf16) {
-      dXa = a.take<float>(bF);
-      dXb = a.take<float>(bF);
-      dX0 = a.take<float>(bF);
-      dA = a.take<float>(bkH);
       dG = a.take<float>(bH);
+      for (int j = 0; j < d.n; ++j) {
+        bb[j].dOut = a.take<float>(bF);
+        bb[j].dA = a.take<float>(bkH);
+        bb[j].dX0 = a.take<float>(bF);
+      }
+      dLte = a.take<float>(bF);
+      dh0 = a.take<float>(bF);
     } else {
       tiles = a.take<TransposeTile>(std::max(1, ntiles));
       for (int j = 0; j < d.n; ++j) {
@@ -351,9 +355,8 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
   }
   if (!d.lte) {
     // "w/o LTE": the FDM reads the last Local block's output and writes the
-    // first Global block's input; in BF16 mode its adjoint reads that input's
-    // gradient and writes the last Local block's output gradient and its BF16
-    // copies (the FP32 adjoint sets dY and dXp per step).
+    // first Global block's input; its adjoint reads that input's gradient and
+    // writes the last Local block's output gradient (and its BF16 copies).
     for (int q = 0; q < npar; ++q) {
       par[q].Xp = par[q].S[d.nloc];
       par[q].Y = par[q].S[d.nloc + 1];
@@ -362,16 +365,14 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
   }
   select(0);
   if (!d.lte) {
-    if (bf16) {
-      dY = dLte;
-      if (d.nloc > 0) {
-        dXp = bb[d.nloc - 1].dOut;
-        dXpb = bb[d.nloc - 1].dOutb;
-        dXpbT = bb[d.nloc - 1].dOutbT;
-      } else {
-        dXp = dh0;
-        dXpb = dXpbT = nullptr;
-      }
+    dY = dLte;
+    if (d.nloc > 0) {
+      dXp = bb[d.nloc - 1].dOut;
+      dXpb = bb[d.nloc - 1].dOutb;
+      dXpbT = bb[d.nloc - 1].dOutbT;
+    } else {
+      dXp = dh0;
+      dXpb = dXpbT = nullptr;
     }
   }
   cudaStream_t st = 0;
@@ -436,12 +437,12 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
     if (ntiles) EDPC_CUDA(cudaMemcpyAsync(tiles, th.data(), th.size() * sizeof(TransposeTile), cudaMemcpyHostToDevice, st));
     EDPC_TRY(refresh_bf16_weights(st));
     EDPC_TRY(build_tc_plan());
-    EDPC_CUDA(cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, delayed ? prio_greatest : prio_least));
-    for (auto& e : fork) EDPC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    EDPC_CUDA(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
     EDPC_CUDA(cudaEventCreateWithFlags(&tr_ev, cudaEventDisableTiming));
-    EDPC_CUDA(cudaEventCreateWithFlags(&fdm_join_ev, cudaEventDisableTiming));
   }
+  EDPC_CUDA(cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, delayed ? prio_greatest : prio_least));
+  for (auto& e : fork) EDPC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  EDPC_CUDA(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
+  EDPC_CUDA(cudaEventCreateWithFlags(&fdm_join_ev, cudaEventDisableTiming));
   if (split) {
     EDPC_CUDA(cudaStreamCreateWithPriority(&side_fdm, cudaStreamNonBlocking, prio_least));
     EDPC_CUDA(cudaEventCreateWithFlags(&dx_ev, cudaEventDisableTiming));
@@ -618,24 +619,39 @@ int Model::forward_f32(const StepIO& io, cudaStream_t st) {
   return EDPC_OK;
 }
 
-int Model::block_bwd(int j, const float* dOut, float* dXnew, cudaStream_t st) {
+// The weight gradients and column sums of a layer, which nothing on the step's
+// critical path waits for, run on the side stream; so every gradient they read
+// has a buffer of its own per block.
+int Model::side_f32(const float* dOut, int out, const float* X, int in, size_t w_off, ColsumJobs cj, cudaStream_t st) {
+  EDPC_TRY(fork_side(st));
+  NoPdl scope;
+  if (X) EDPC_TRY(linear_dw(dOut, d.b, out, X, in, w_off, side));
+  if (cj.n) EDPC_CUDA(launch_colsum(cj, side));
+  return EDPC_OK;
+}
+
+int Model::block_bwd(int j, float* dXnew, cudaStream_t st) {
   const BlockOff& o = po.blk[j];
   BlockAct& a = ba[j];
+  BlockBf16& q = bb[j];
   const int kH = d.k * d.H;
   // Eq. 13: out = G Wo^T + co + X
-  EDPC_TRY(linear_dw(dOut, d.b, d.F, a.G, d.H, o.Wo, st));
-  EDPC_CUDA(launch_colsum(dOut, nullptr, d.b, d.F, d.F, G + o.co, st));
-  EDPC_TRY(linear_dx(dOut, d.b, d.F, o.Wo, d.H, dG, st));
+  EDPC_TRY(side_f32(q.dOut, d.F, a.G, d.H, o.Wo, ColsumJobs{}, st));
+  EDPC_TRY(linear_dx(q.dOut, d.b, d.F, o.Wo, d.H, dG, st));
   // Eqs. 11-12: G = GELU(prod X_i)
-  EDPC_CUDA(launch_branch_gelu_bwd(dG, a.A, d.b, d.H, d.k, dA, st));
+  EDPC_CUDA(launch_branch_gelu_bwd(dG, a.A, d.b, d.H, d.k, q.dA, st));
   // Eq. 10: X_i = X0 W_i^T + c_i
-  EDPC_TRY(linear_dw(dA, d.b, kH, a.X0, d.F, o.W, st));
-  EDPC_CUDA(launch_colsum(dA, nullptr, d.b, kH, kH, G + o.c, st));
-  EDPC_TRY(linear_dx(dA, d.b, kH, o.W, d.F, dX0, st));
+  EDPC_TRY(side_f32(q.dA, kH, a.X0, d.F, o.W, ColsumJobs{}, st));
+  EDPC_TRY(linear_dx(q.dA, d.b, kH, o.W, d.F, q.dX0, st));
+  ColsumJobs cj{};
+  cj.job[0] = {q.dOut, nullptr, d.b, d.F, d.F, G + o.co};
+  cj.job[1] = {q.dA, nullptr, d.b, kH, kH, G + o.c};
+  cj.job[2] = {q.dX0, a.xhat, d.b, d.F, d.F, G + o.ln_g};
+  cj.job[3] = {q.dX0, nullptr, d.b, d.F, d.F, G + o.ln_b};
+  cj.n = 4;
+  EDPC_TRY(side_f32(nullptr, 0, nullptr, 0, 0, cj, st));
   // Eq. 9: X0 = g * xhat + beta, plus the residual path of Eq. 13
-  EDPC_CUDA(launch_colsum(dX0, a.xhat, d.b, d.F, d.F, G + o.ln_g, st));
-  EDPC_CUDA(launch_colsum(dX0, nullptr, d.b, d.F, d.F, G + o.ln_b, st));
-  EDPC_CUDA(launch_ln_bwd(dX0, a.xhat, a.rstd, P + o.ln_g, dOut, dXnew, d.b, d.F, st));
+  EDPC_CUDA(launch_ln_bwd(q.dX0, a.xhat, a.rstd, P + o.ln_g, q.dOut, dXnew, d.b, d.F, st));
   return EDPC_OK;
 }
 
@@ -712,39 +728,35 @@ int Model::fdm_bwd_call(const StepIO& io, cudaStream_t st) {
 }
 
 int Model::backward_f32(const StepIO& io, cudaStream_t st) {
-  const float* head_in = S[d.n + 1];
-  EDPC_TRY(linear_dw(dz, d.b, 256, head_in, d.F, po.Wh, st));
-  EDPC_CUDA(launch_colsum(dz, nullptr, d.b, 256, 256, G + po.bh, st));
-  EDPC_TRY(linear_dx(dz, d.b, 256, po.Wh, d.F, dXa, st));
-  float* cur = dXa;
-  float* nxt = dXb;
-  for (int j = d.n - 1; j >= d.nloc; --j) {
-    EDPC_TRY(block_bwd(j, cur, nxt, st));
-    std::swap(cur, nxt);
-  }
-  if (d.lte) {
+  nfork_ = 0;
+  auto one = [&](const float* X, int cols, size_t off) {
+    ColsumJobs cj{};
+    cj.job[0] = {X, nullptr, d.b, cols, cols, G + off};
+    cj.n = 1;
+    return cj;
+  };
+  EDPC_TRY(side_f32(dz, 256, S[d.n + 1], d.F, po.Wh, one(dz, 256, po.bh), st));
+  EDPC_TRY(linear_dx(dz, d.b, 256, po.Wh, d.F, bb[d.n - 1].dOut, st));
+  auto middle = [&]() -> int {  // between the Global and the Local blocks
+    if (!d.lte) return fdm_bwd_joined(io, st);  // the FDM's adjoint alone: dLte -> dXp
     // LTE up (Eq. 16)
-    EDPC_TRY(linear_dw(cur, d.b, d.F, Y, d.Fp, po.W2, st));
-    EDPC_CUDA(launch_colsum(cur, nullptr, d.b, d.F, d.F, G + po.b2, st));
-    EDPC_TRY(linear_dx(cur, d.b, d.F, po.W2, d.Fp, dY, st));
+    EDPC_TRY(side_f32(dLte, d.F, Y, d.Fp, po.W2, one(dLte, d.F, po.b2), st));
+    EDPC_TRY(linear_dx(dLte, d.b, d.F, po.W2, d.Fp, dY, st));
     // FDM (Eq. 15): adjoint fused with the FDM's Adam update
-    EDPC_TRY(fdm_bwd_call(io, st));
+    EDPC_TRY(fdm_bwd_joined(io, st));
     // LTE down (Eq. 14)
-    EDPC_TRY(linear_dw(dXp, d.b, d.Fp, S[d.nloc], d.F, po.W1, st));
-    EDPC_CUDA(launch_colsum(dXp, nullptr, d.b, d.Fp, d.Fp, G + po.b1, st));
-    EDPC_TRY(linear_dx(dXp, d.b, d.Fp, po.W1, d.F, cur, st));
-  } else {
-    // w/o LTE: the FDM's adjoint maps the gradient of S[nloc + 1] to that of S[nloc]
-    dY = cur;
-    dXp = nxt;
-    EDPC_TRY(fdm_bwd_call(io, st));
-    std::swap(cur, nxt);
+    EDPC_TRY(side_f32(dXp, d.Fp, S[d.nloc], d.F, po.W1, one(dXp, d.Fp, po.b1), st));
+    return linear_dx(dXp, d.b, d.Fp, po.W1, d.F, d.nloc > 0 ? bb[d.nloc - 1].dOut : dh0, st);
+  };
+  for (int j = d.n - 1; j >= 0; --j) {
+    if (j == d.nloc - 1) EDPC_TRY(middle());
+    EDPC_TRY(block_bwd(j, j == d.nloc ? dLte : (j == 0 ? dh0 : bb[j - 1].dOut), st));
   }
-  for (int j = d.nloc - 1; j >= 0; --j) {
-    EDPC_TRY(block_bwd(j, cur, nxt, st));
-    std::swap(cur, nxt);
-  }
-  EDPC_CUDA(launch_embed_bwd(ctx, cur, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, st));
+  if (d.nloc == 0) EDPC_TRY(middle());
+  EDPC_CUDA(launch_embed_bwd(ctx, dh0, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, st));
+  // join the side stream
+  EDPC_CUDA(cudaEventRecord(join_ev, side));
+  EDPC_CUDA(cudaStreamWaitEvent(st, join_ev, 0));
   return EDPC_OK;
 }
 
@@ -1481,6 +1493,7 @@ int Model::adam(cudaStream_t st) {
     NoPdl scope;  // follows the join of the side stream
     EDPC_CUDA(launch_adam_bf16(P, G, M, V, Pb, np_all, ctl, st));
   } else {
+    NoPdl scope;
     EDPC_CUDA(launch_adam(P, G, M, V, nparam, ctl, st));
   }
   return EDPC_OK;

@@ -18,7 +18,7 @@ struct BlockAct {
   float* G;     // b x H  GELU(X_fused) (Eq. 12), FP32 path
 };
 
-// BF16-path buffers of one MBRB block. "T" buffers are transposed copies
+// Gradients of one MBRB block (FP32, both paths) and its BF16-path buffers. "T" buffers are transposed copies
 // [feature][ldT], the K-major operands of the dW GEMMs (contraction over streams).
 struct BlockBf16 {
   __nv_bfloat16 *X0b, *X0bT;      // LN output
@@ -49,7 +49,7 @@ class Model {
   float* S[kMaxBlocks + 2] = {};          // residual-stream stages, b x F
   BlockAct ba[kMaxBlocks] = {};
   float *Xp = nullptr, *Y = nullptr, *z = nullptr, *p = nullptr, *dz = nullptr;
-  float *dXa = nullptr, *dXb = nullptr, *dX0 = nullptr, *dA = nullptr, *dG = nullptr;
+  float* dG = nullptr;                    // FP32 path: gradient w.r.t. a block's GELU output
   float *dY = nullptr, *dXp = nullptr;
   float* emb_part = nullptr;              // embedding-adjoint chunk partials (many positions)
   unsigned* emb_cnt = nullptr;            // their arrival counters, one per byte value
@@ -218,7 +218,8 @@ class Model {
   int nfork_ = 0;
   // FP32 path
   int block_fwd(int j, const float* Xin, float* Xout, cudaStream_t st);
-  int block_bwd(int j, const float* dOut, float* dXnew, cudaStream_t st);
+  int block_bwd(int j, float* dXnew, cudaStream_t st);
+  int side_f32(const float* dOut, int out, const float* X, int in, size_t w_off, ColsumJobs cj, cudaStream_t st);
   int forward_f32(const StepIO& io, cudaStream_t st);
   int backward_f32(const StepIO& io, cudaStream_t st);
   int linear_fwd(const float* X, int rows, int in, size_t w_off, size_t b_off, int out, const float* resid, float* Yo,

@@ -193,37 +193,57 @@ cudaError_t launch_branch_gelu_bwd(const float* dG, const float* A, int b, int H
 }
 
 // ============================================================================================
-// Column sums over rows (bias and LN-affine gradients), fixed order:
-// warp w sums rows w, w+8, ... for 32 columns; then warps are added in order.
+// Column sums over rows of the FP32 path (bias and LN-affine gradients), all of
+// a block's tensors in one launch, fixed order: warp w sums rows w, w+8, ...
+// for 32 columns; then warps are added in order.
 // ============================================================================================
-__global__ void colsum_kernel(const float* __restrict__ X, const float* __restrict__ Y, int rows, int cols,
-                              int ld, float* __restrict__ out) {
+__global__ void __launch_bounds__(256) colsum_kernel(ColsumJobs jobs) {
   pdl_wait();
   pdl_launch();
   __shared__ float part[8][33];
+  int t = blockIdx.x, j = 0;
+  while (j < jobs.n - 1 && t >= (jobs.job[j].cols + 31) / 32) {
+    t -= (jobs.job[j].cols + 31) / 32;
+    ++j;
+  }
+  const ColsumJob jb = jobs.job[j];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * 32 + lane;
+  const int c = t * 32 + lane;
   float s = 0.f;
-  if (c < cols) {
-    if (Y) {
-      for (int r = w; r < rows; r += 8) s += X[(size_t)r * ld + c] * Y[(size_t)r * ld + c];
-    } else {
-      for (int r = w; r < rows; r += 8) s += X[(size_t)r * ld + c];
+  if (c < jb.cols) {
+    // the rows' loads go out sixteen at a time; the adds keep their order
+    constexpr int U = 16;
+    const size_t ld = (size_t)jb.ld;
+    const float* x = jb.X + (size_t)w * ld + c;
+    const float* y = jb.Y ? jb.Y + (size_t)w * ld + c : nullptr;
+    for (int r = w; r < jb.rows; r += 8 * U) {
+      const size_t o = (size_t)(r - w) * ld;
+      float vx[U], vy[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const bool in = r + 8 * q < jb.rows;
+        vx[q] = in ? x[o + 8 * q * ld] : 0.f;
+        vy[q] = in && y ? y[o + 8 * q * ld] : 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (r + 8 * q < jb.rows) s = y ? fmaf(vx[q], vy[q], s) : s + vx[q];
     }
   }
   part[w][lane] = s;
   __syncthreads();
-  if (w == 0 && c < cols) {
-    float t = part[0][lane];
+  if (w == 0 && c < jb.cols) {
+    float v = part[0][lane];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) t += part[i][lane];
-    out[c] = t;
+    for (int i = 1; i < 8; ++i) v += part[i][lane];
+    jb.out[c] = v;
   }
 }
 
-cudaError_t launch_colsum(const float* X, const float* Y, int rows, int cols, int ld, float* out,
-                          cudaStream_t st) {
-  return launch_k(colsum_kernel, dim3(div_up(cols, 32)), dim3(256), 0, st, X, Y, rows, cols, ld, out);
+cudaError_t launch_colsum(const ColsumJobs& jobs, cudaStream_t st) {
+  int tiles = 0;
+  for (int j = 0; j < jobs.n; ++j) tiles += div_up(jobs.job[j].cols, 32);
+  return launch_k(colsum_kernel, dim3(tiles), dim3(256), 0, st, jobs);
 }
 
 // ============================================================================================

@@ -72,9 +72,10 @@ cudaError_t launch_head(const HeadArgs& a, cudaStream_t st);
 // ---- backward -----------------------------------------------------------------------------
 cudaError_t launch_branch_gelu_bwd(const float* dG, const float* A, int b, int H, int k, float* dA,
                                    cudaStream_t st);
-// out[c] = sum_r X[r][c] (or sum_r X[r][c] * Y[r][c] when Y != nullptr), fixed order.
-cudaError_t launch_colsum(const float* X, const float* Y, int rows, int cols, int ld, float* out,
-                          cudaStream_t st);
+// out[c] = sum_r X[r][c] (or sum_r X[r][c] * Y[r][c] when Y != nullptr) for each
+// job, fixed order (the chunk fields of jobs unused).
+struct ColsumJobs;
+cudaError_t launch_colsum(const ColsumJobs& jobs, cudaStream_t st);
 // dX = dRes + LN backward of dX0.
 cudaError_t launch_ln_bwd(const float* dX0, const float* xhat, const float* rstd, const float* g,
                           const float* dRes, float* dX, int b, int F, cudaStream_t st);
