@@ -1,16 +1,18 @@
 // BF16 / FP8 GEMM on the 5th-generation tensor cores (sm_103a).
 //
 // One CTA computes a 128 x BN tile of C = A B^T:
-//   warp 0 (one lane)  issues TMA loads of 128-byte-wide A (128 rows) and B
+//   warp 8 (one lane)  issues TMA loads of 128-byte-wide A (128 rows) and B
 //                      (BN rows) tiles (64 BF16 or 128 FP8 elements of K,
 //                      128-byte swizzle) into a STAGES-deep ring;
-//   warp 1 (one lane)  issues tcgen05.mma (M=128, N=BN; kind::f16 with K=16
+//   warp 9 (one lane)  issues tcgen05.mma (M=128, N=BN; kind::f16 with K=16
 //                      for BF16, kind::f8f6f4 with K=32 for FP8 e4m3; FP32
 //                      accumulation) into a TMEM accumulator and commits each
-//                      stage back to its "empty" barrier;
-//   warp 2             allocates / frees the TMEM columns;
-//   warps 0-3          drain TMEM with tcgen05.ld (warp w owns lanes 32w..32w+31,
-//                      i.e. tile rows) and run the fused epilogue.
+//                      stage back to its "empty" barrier, and allocates / frees
+//                      the TMEM columns;
+//   warps 0-7          run the fused epilogue (tc_epilogue8): its accumulator-
+//                      independent part beside the main loop, then TMEM by
+//                      tcgen05.ld (warp w: rows 32 (w & 3) .., 16 of every 32
+//                      columns).
 // The MMA order over K is fixed, so results are deterministic.
 // Barrier set-up, TMEM allocation and tensor-map prefetch run before the
 // programmatic-dependent-launch wait, overlapping the previous kernel's tail.
@@ -45,12 +47,14 @@ constexpr size_t smem_bytes() {
   return 1024 /*alignment slack*/ + (size_t)stages_for<BN>() * (BM * BKB + BN * BKB) + 256;
 }
 
+constexpr int kTcThreads = kEpiThreads + 64;
+
 // KB: branch count k (TC_BRANCH, TC_BRANCH_BWD; 1 otherwise). In TC_BRANCH mode
 // the N tile holds k sections of SW = BN / k hidden units each.
 // GR: grouped mode (the tile list, or each group's K range; see TcGemm). The
 // other instantiations carry none of its code.
 template <int BN, int MODE, int KB, bool F8, bool GR>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTcThreads, BN <= 64 ? 1 : 2)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                    const __grid_constant__ CUtensorMap tmc, const __grid_constant__ CUtensorMap tmcb, const TcEpi e) {
   extern __shared__ uint8_t smem_raw[];
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(128, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&ta)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tb)) : "memory");
   }
-  if (warp == 2) {
+  if (warp == 9) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)tmem_cols<BN>()));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -132,16 +136,34 @@ __global__ void __launch_bounds__(128, 1)
     }
   };
   const int npre = e.b_early ? (nk < STAGES ? nk : STAGES) : 0;
-  if (warp == 0 && lane == 0) {
+  if (warp == 8 && lane == 0) {
     for (int kb = 0; kb < npre; ++kb) {
       mbar_expect_tx(&full[kb], A_BYTES + B_BYTES);
       load_b(kb, kb);
     }
   }
+  // The epilogue's view of the problem; grouped mode: the tile's row bound, its
+  // group's bias or gradient output.
+  TcEpi eg = e;
+  if constexpr (GR) {
+    eg.M = mend;
+    eg.rlim = mend;
+    if (e.mt && e.bias) eg.bias = e.bias + (long long)grp * e.gs;
+    if (e.gk) eg.C = e.C + (long long)grp * e.gs;
+  }
+  // The pipeline's A stages are idle by then: they hold the epilogue's slots.
+  constexpr int SLOTS = STAGES * A_BYTES / kEpiSlot;
+  static_assert(SLOTS >= 1, "A stages hold the epilogue staging");
+  const int tr = (warp & 3) * 32 + lane;  // tile row of an epilogue thread
+  const Epi8 x{eg, &tmc, &tmcb, sA, m0, n0, m0 + tr, tr, warp >> 2, lane, warp, (int)threadIdx.x, m0 + tr < eg.M};
+  EpiPre<MODE, KB> pre;
+  // The bias, the residual and the saved branch outputs were written at least
+  // two launches earlier: fetched ahead of the dependent-launch wait.
+  if (warp < 8) epi_fetch<MODE, KB>(x, 0, pre);
   pdl_wait();
   pdl_launch();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 8 && lane == 0) {
     // TMA producer
     for (int kb = 0; kb < nk; ++kb) {
       const int s = kb % STAGES;
@@ -153,7 +175,7 @@ __global__ void __launch_bounds__(128, 1)
       }
       tma_load_2d(sA + s * A_BYTES, &ta, kel0 + (kb_lo + kb) * BK, m0, &full[s]);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 9 && lane == 0) {
     // MMA issuer
     constexpr uint32_t idesc = F8 ? idesc_e4m3(BN) : idesc_bf16(BN);
     for (int kb = 0; kb < nk; ++kb) {
@@ -176,31 +198,17 @@ __global__ void __launch_bounds__(128, 1)
   }
   __syncwarp();
 
-  // Epilogue: thread (warp w, lane l) owns tile row 32w + l. The TMEM loads are
-  // warp-collective, so the wait result is made CTA-uniform first.
+  if (warp < 8) epi_early<MODE, KB>(pre);
+  // The TMEM loads are warp-collective, so the wait result is made CTA-uniform first.
   const bool ok = __syncthreads_and(mbar_wait(done, 0, abort_flag) ? 1 : 0) != 0;
   tc_fence_after();
-  // The pipeline's A stages are idle now: reuse them to stage the transposed
-  // stores (8 KB) and the TMA stores (6 KB per warp).
-  static_assert(STAGES * A_BYTES >= 8192 + kStageOut, "A stages hold the epilogue staging");
-  if (ok) {
-    const EpiOut o{&tmc, &tmcb, sA + 8192 + warp * kStageOutWarp, m0 + warp * 32, lane};
-    if constexpr (GR) {
-      // grouped mode: the tile's row bound, its group's bias or gradient output
-      TcEpi eg = e;
-      eg.M = mend;
-      eg.rlim = mend;
-      if (e.mt && e.bias) eg.bias = e.bias + (long long)grp * e.gs;
-      if (e.gk) eg.C = e.C + (long long)grp * e.gs;
-      tc_epilogue<BN, MODE, KB, F8>(eg, tmem + ((uint32_t)(warp * 32) << 16), m0, n0, 0, 1, 0,
-                                    reinterpret_cast<__nv_bfloat16*>(sA),
-                                    reinterpret_cast<volatile int*>(tmem_slot + 2), threadIdx.x, threadIdx.x, o);
-    } else {
-      tc_epilogue<BN, MODE, KB, F8>(e, tmem + ((uint32_t)(warp * 32) << 16), m0, n0, blockIdx.z, gridDim.z,
-                                    blockIdx.y * gridDim.x + blockIdx.x, reinterpret_cast<__nv_bfloat16*>(sA),
-                                    reinterpret_cast<volatile int*>(tmem_slot + 2), threadIdx.x, threadIdx.x, o);
-    }
-    tma_st_drain(lane);
+  if (ok && warp < 8) {
+    tc_epilogue8<BN, MODE, KB, F8, SLOTS>(x, tmem + ((uint32_t)((warp & 3) * 32) << 16), GR ? 0 : blockIdx.z,
+                                          GR ? 1 : gridDim.z, blockIdx.y * gridDim.x + blockIdx.x,
+                                          reinterpret_cast<volatile int*>(tmem_slot + 2), pre);
+    // the staging must outlive the stores' reads; the grid's end makes their writes visible
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncwarp();
   }
   if (!ok && threadIdx.x == 0 && e.err) atomicOr(e.err, kErrTcTimeout);
   tc_fence_before();
@@ -212,7 +220,7 @@ __global__ void __launch_bounds__(128, 1)
         if (mbar_try_wait(&full[s], 0) || mbar_try_wait(&full[s], 1)) break;
     }
   }
-  if (warp == 2) {
+  if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"((uint32_t)tmem_cols<BN>()));
@@ -236,7 +244,7 @@ cudaError_t launch_bn_mode_g(const TcGemm& g, cudaStream_t st) {
   constexpr int SW = (MODE == TC_BRANCH) ? BN / KB : BN;
   const int ntile = (MODE == TC_BRANCH) ? (g.H + SW - 1) / SW : (g.N + BN - 1) / BN;
   dim3 grid(ntile, g.mt ? g.nmt : (g.M + BM - 1) / BM, g.gk ? g.ngk : (g.splitk > 1 ? g.splitk : 1));
-  return launch_k(k, grid, dim3(128), smem_bytes<BN>(), st, g.ta, g.tb, g.tmc, g.tmcb, e);
+  return launch_k(k, grid, dim3(kTcThreads), smem_bytes<BN>(), st, g.ta, g.tb, g.tmc, g.tmcb, e);
 }
 
 // Grouped launches (BF16 only) use the GR instantiation.
@@ -323,7 +331,7 @@ int tc_build_out_maps(TcGemm* g) {
     if ((reinterpret_cast<uintptr_t>(base) & 15) || (((size_t)ld * esize) & 15)) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)g->M};
     cuuint64_t strides[1] = {(cuuint64_t)ld * esize};
-    cuuint32_t box[2] = {32, 32};
+    cuuint32_t box[2] = {g->persistent ? 32u : 16u, 32};  // the kernel's chunk: 32 rows x 32 or 16 columns
     cuuint32_t estr[2] = {1, 1};
     return enc(tm, dt, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -334,8 +342,10 @@ int tc_build_out_maps(TcGemm* g) {
   // split-K partials and their sums, and grouped weight gradients (one output
   // base per group), keep direct stores
   if (g->splitk <= 1 && cols_ok && !g->gk) {
-    g->has_tmc = build(&g->tmc, g->C, wc, g->ldc, 4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, CU_TENSOR_MAP_SWIZZLE_128B);
-    g->has_tmcb = build(&g->tmcb, g->Cb, wcb, g->ldcb, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_64B);
+    g->has_tmc = build(&g->tmc, g->C, wc, g->ldc, 4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                       g->persistent ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+    g->has_tmcb = build(&g->tmcb, g->Cb, wcb, g->ldcb, 2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                        g->persistent ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
   }
   return EDPC_OK;
 }

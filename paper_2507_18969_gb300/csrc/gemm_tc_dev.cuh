@@ -221,9 +221,11 @@ __device__ __forceinline__ void store_row32(const float (&v)[32], bool rok, int 
   }
 }
 
-// Barrier of the 128 epilogue threads (named barrier 1; the whole CTA in the
-// one-tile kernel, warps 2-5 in the persistent one).
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// Barrier of the epilogue threads (named barrier 1): 256 in the one-tile kernel
+// (warps 0-7), 128 in the persistent one (warps 2-5).
+template <int NT>
+__device__ __forceinline__ void epi_sync_n() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
+__device__ __forceinline__ void epi_sync() { epi_sync_n<128>(); }
 // CTA-uniform AND of a predicate over the 128 epilogue threads.
 __device__ __forceinline__ bool epi_and(bool p) {
   uint32_t r;
@@ -348,19 +350,19 @@ static_assert(tmem_cols<256>() == 256, "N tiles above 256 do not fit one MMA");
 // 0, 1, ..., S - 1 in that order and writes C, then zeroes the counter.
 // Collective over the epilogue threads; `flag` is a shared-memory word; S is
 // the split count and tile the output tile's counter index.
-template <int BN>
+template <int BN, int NT>
 __device__ __forceinline__ void splitk_finish(const TcEpi& e, int m0, int n0, int S, int tile, volatile int* flag,
                                               int et) {
-  epi_sync();
+  epi_sync_n<NT>();
   if (et == 0) *flag = (atomicAdd(&e.cnt[tile], 1u) == (unsigned)(S - 1)) ? 1 : 0;
-  epi_sync();
+  epi_sync_n<NT>();
   if (!*flag) return;
   __threadfence();
   const size_t plane = (size_t)e.M * e.N;
   const bool vec = (e.N % 4 == 0) && (e.ldc % 4 == 0) && ((reinterpret_cast<uintptr_t>(e.C) & 15) == 0) &&
                    ((reinterpret_cast<uintptr_t>(e.ws) & 15) == 0);
   constexpr int C4 = BN / 4;
-  for (int idx = et; idx < BM * C4; idx += 128) {
+  for (int idx = et; idx < BM * C4; idx += NT) {
     const int r = idx / C4, c = (idx % C4) * 4;
     const int gm = m0 + r, gn = n0 + c;
     if (gm >= e.M || gn >= e.N) continue;
@@ -416,7 +418,7 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t trow, int m
       store_row32(v, rok, n0 + c0, e.N, wrow, nullptr);
     }
     __threadfence();
-    splitk_finish<BN>(e, m0, n0, S, tile, flag, et);
+    splitk_finish<BN, 128>(e, m0, n0, S, tile, flag, et);
   } else if (MODE == TC_PLAIN) {
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
@@ -512,6 +514,322 @@ __device__ __forceinline__ void tc_epilogue(const TcEpi& e, uint32_t trow, int m
         store_T32(dd, sT, m0, colb + hb, colb + e.H, e.CbT, e.ldct, r, et, e.rlim);
       }
     }
+  }
+}
+
+// ---- the one-tile kernel's epilogue -----------------------------------------------------------
+// Eight warps share the 128 x BN tile: warp w reads TMEM lanes 32 (w & 3) .. and
+// 16 of every 32 columns (half w >> 2). What bounds the small launches is the
+// latency of this tail (32 to 64 CTAs, one tile each, nothing to overlap it
+// with), so everything that does not depend on the accumulator (bias, residual,
+// saved branch outputs, GELU's derivative) is fetched and computed for the
+// first chunk while the main loop runs, each output chunk has staging of its
+// own (kEpiSlot bytes per chunk in the idle A stages), and the CTA leaves once
+// the stores have read it. With four warps of 32 columns each, loads after the
+// main loop and one staging area, the branch adjoint of 512 x 256 outputs took
+// 11.3 us of the step and the branch GEMM 7.5; now 6.1 and 5.7.
+constexpr int kEpiThreads = 256;
+constexpr int kEpiStgWarp = 3072;                            // 32 x 16 FP32, then 32 x 16 BF16
+constexpr int kEpiSlot = 8192 + 8 * kEpiStgWarp;             // transposed chunk, then the warps' staging
+
+__device__ __forceinline__ void epi_sync8() { epi_sync_n<kEpiThreads>(); }
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// 16 consecutive FP32 values src[n0 ..) (0 at or beyond N; vectorised when whole and aligned).
+__device__ __forceinline__ void load16(const float* src, int n0, int N, float (&v)[16]) {
+  if (n0 + 16 <= N && ((reinterpret_cast<uintptr_t>(src + n0) & 15) == 0)) {
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(src + n0 + j);
+      v[j] = q.x;
+      v[j + 1] = q.y;
+      v[j + 2] = q.z;
+      v[j + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = (n0 + j < N) ? src[n0 + j] : 0.f;
+  }
+}
+
+__device__ __forceinline__ uint4 pack8(const float* v) {
+  __align__(16) __nv_bfloat162 h[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+  return *reinterpret_cast<const uint4*>(h);
+}
+
+struct Epi8 {
+  const TcEpi& e;
+  const CUtensorMap *tmc, *tmcb;  // boxes of 32 rows x 16 columns
+  uint8_t* base;                  // NS slots
+  int m0, n0;
+  int row, r, half, lane, warp, et;
+  bool rok;
+};
+
+// 16 columns [cb, cb + 16) of the warp's 32 rows, of the logical region of
+// width w that starts at column `base` of C and Cb: whole chunks by TMA store
+// from staging (64-byte FP32 rows with the 64-byte swizzle, 32-byte BF16 rows
+// with the 32-byte one), others by direct stores.
+__device__ __forceinline__ void put_chunk(const Epi8& x, uint8_t* stg, const float (&v)[16], int base, int cb, int w,
+                                          float* C, __nv_bfloat16* Cb) {
+  const TcEpi& e = x.e;
+  const int r0 = x.m0 + (x.warp & 3) * 32;
+  const bool whole = cb + 16 <= w && r0 + 32 <= e.M;
+  const bool tc = C && whole && e.tma_c, tb = Cb && whole && e.tma_cb;
+  if (tc) {
+    uint8_t* rp = stg + x.lane * 64;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<float4*>(rp + ((j ^ ((x.lane >> 1) & 3)) << 4)) =
+          make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+  } else if (C && x.rok) {
+    float* p = C + (size_t)x.row * e.ldc + base + cb;
+    if (cb + 16 <= w && ((reinterpret_cast<uintptr_t>(p) & 15) == 0)) {
+#pragma unroll
+      for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(p + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (cb + j < w) p[j] = v[j];
+    }
+  }
+  if (tb) {
+    uint8_t* rp = stg + 2048 + x.lane * 32;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) *reinterpret_cast<uint4*>(rp + ((j ^ ((x.lane >> 2) & 1)) << 4)) = pack8(v + 8 * j);
+  } else if (Cb && x.rok) {
+    __nv_bfloat16* p = Cb + (size_t)x.row * e.ldcb + base + cb;
+    if (cb + 16 <= w && ((reinterpret_cast<uintptr_t>(p) & 15) == 0)) {
+#pragma unroll
+      for (int j = 0; j < 16; j += 8) *reinterpret_cast<uint4*>(p + j) = pack8(v + j);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (cb + j < w) p[j] = __float2bfloat16_rn(v[j]);
+    }
+  }
+  if (tc || tb) {  // warp-uniform
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (x.lane == 0) {
+      if (tc)
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                         reinterpret_cast<uint64_t>(x.tmc)),
+                     "r"(base + cb), "r"(r0), "r"(smem_u32(stg))
+                     : "memory");
+      if (tb)
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                         reinterpret_cast<uint64_t>(x.tmcb)),
+                     "r"(base + cb), "r"(r0), "r"(smem_u32(stg + 2048))
+                     : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+  }
+}
+
+// The thread's 16 columns into the transposed chunk (column-major, 128 rows a column).
+__device__ __forceinline__ void put_T(const Epi8& x, __nv_bfloat16* sT, const float (&v)[16]) {
+#pragma unroll
+  for (int c = 0; c < 16; ++c) sT[(16 * x.half + c) * 128 + x.r] = __float2bfloat16_rn(v[c]);
+}
+// 32 columns of 128 rows as 16-byte runs to CT[(c0 + c) * ldct + m0 + row] (columns below N, runs inside ldct).
+__device__ __forceinline__ void flush_T(const Epi8& x, const __nv_bfloat16* sT, int c0, int N) {
+  const TcEpi& e = x.e;
+#pragma unroll
+  for (int idx = x.et; idx < 32 * 16; idx += kEpiThreads) {
+    const int c = idx >> 4, seg = idx & 15;
+    const int row0 = x.m0 + seg * 8;
+    if (c0 + c < N && row0 + 8 <= e.ldct && row0 + 8 <= e.rlim)
+      *reinterpret_cast<uint4*>(e.CbT + (size_t)(c0 + c) * e.ldct + row0) =
+          *reinterpret_cast<const uint4*>(sT + c * 128 + seg * 8);
+  }
+}
+
+// What the first chunk needs besides the accumulator.
+template <int MODE, int KB>
+struct EpiPre {
+  float a[MODE == TC_PLAIN ? 1 : KB][16];  // bias (PLAIN: of the chunk; BRANCH: of every section) or branch outputs
+  float b[16];                             // PLAIN: residual; BRANCH_BWD: GELU'(product)
+};
+
+template <int MODE, int KB>
+__device__ __forceinline__ void epi_fetch(const Epi8& x, int c0, EpiPre<MODE, KB>& p) {
+  const TcEpi& e = x.e;
+  const int cb = x.n0 + c0 + 16 * x.half;
+  if (MODE == TC_PLAIN) {
+    if (e.bias) load16(e.bias, cb, e.N, p.a[0]);
+    if (e.R && x.rok) load16(e.R + (size_t)x.row * e.ldr, cb, e.N, p.b);
+  } else if (MODE == TC_BRANCH) {
+#pragma unroll
+    for (int i = 0; i < KB; ++i) load16(e.bias + i * e.H, cb, e.H, p.a[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      if (x.rok) {
+        load16(e.Aux + (size_t)x.row * e.ldaux + i * e.H, cb, e.H, p.a[i]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) p.a[i][j] = 0.f;
+      }
+    }
+  }
+}
+template <int MODE, int KB>
+__device__ __forceinline__ void epi_early(EpiPre<MODE, KB>& p) {
+  if (MODE == TC_BRANCH_BWD) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      float xf = 1.f;
+#pragma unroll
+      for (int i = 0; i < KB; ++i) xf *= p.a[i][j];
+      p.b[j] = gelu_grad_f(xf);
+    }
+  }
+}
+
+// trow: TMEM address of the warp's lanes and the accumulator's first column.
+// NS slots of kEpiSlot bytes at x.base; p: the first chunk's epi_fetch + epi_early.
+template <int BN, int MODE, int KB, bool F8, int NS>
+__device__ __forceinline__ void tc_epilogue8(const Epi8& x, uint32_t trow, int z, int S, int tile, volatile int* flag,
+                                             EpiPre<MODE, KB>& p) {
+  const TcEpi& e = x.e;
+  constexpr int SECTIONS = (MODE == TC_BRANCH) ? KB : 1;
+  constexpr int SW = BN / SECTIONS;
+  // FP8: undo the operands' power-of-two scales (exact)
+  const float sc = F8 ? e.inv_a[0] * e.inv_b[0] : 1.f;
+  int us = 0, ut = 0;
+  auto staging = [&]() -> uint8_t* {  // the warp's staging of the next slot
+    if (us >= NS) {
+      if (x.lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      __syncwarp();
+    }
+    return x.base + (us++ % NS) * kEpiSlot + 8192 + x.warp * kEpiStgWarp;
+  };
+  auto transp = [&]() -> __nv_bfloat16* {  // the next slot's transposed chunk
+    if (ut >= NS) epi_sync8();
+    return reinterpret_cast<__nv_bfloat16*>(x.base + (ut++ % NS) * kEpiSlot);
+  };
+  auto acc = [&](int col, float (&v)[16]) {
+    tmem_ld16(trow + (uint32_t)col, v);
+    if (F8) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] *= sc;
+    }
+  };
+#pragma unroll 1
+  for (int c0 = 0; c0 < SW; c0 += 32) {
+    const int lc = c0 + 16 * x.half;  // the thread's first column within the tile (section)
+    const int cb = x.n0 + lc;
+    float v[16];
+    if (MODE == TC_PLAIN && S > 1) {
+      // split-K: FP32 partial tile -> ws[z]
+      acc(lc, v);
+      if (x.rok) {
+        float* w = e.ws + ((size_t)z * e.M + x.row) * e.N + cb;
+        if (cb + 16 <= e.N && ((reinterpret_cast<uintptr_t>(w) & 15) == 0)) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 4)
+            *reinterpret_cast<float4*>(w + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (cb + j < e.N) w[j] = v[j];
+        }
+      }
+      continue;
+    }
+    if (c0 > 0) {
+      epi_fetch<MODE, KB>(x, c0, p);
+      epi_early<MODE, KB>(p);
+    }
+    if (MODE == TC_PLAIN) {
+      acc(lc, v);
+      if (e.bias) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += p.a[0][j];
+      }
+      if (e.R && x.rok) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += p.b[j];
+      }
+      put_chunk(x, staging(), v, 0, cb, e.N, e.C, e.Cb);
+      if (e.CbT) {
+        __nv_bfloat16* sT = transp();
+        put_T(x, sT, v);
+        epi_sync8();
+        flush_T(x, sT, x.n0 + c0, e.N);
+      }
+    } else if (MODE == TC_BRANCH) {
+      // X_i of hidden units cb + j, then G = GELU(prod X_i); section i is TMEM columns [i*SW, i*SW + SW)
+      float g[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) g[j] = 1.f;
+#pragma unroll
+      for (int i = 0; i < SECTIONS; ++i) {
+        acc(i * SW + lc, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          if (cb + j < e.H) v[j] += p.a[i][j];
+          g[j] *= v[j];
+        }
+        put_chunk(x, staging(), v, i * e.H, cb, e.H, e.C, nullptr);  // X_i, kept for the adjoint
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) g[j] = gelu_f(g[j]);
+      __nv_bfloat16* sT = transp();
+      put_T(x, sT, g);
+      put_chunk(x, staging(), g, 0, cb, e.H, nullptr, e.Cb);
+      epi_sync8();
+      flush_T(x, sT, x.n0 + c0, e.H);
+    } else {
+      // dG of hidden units cb + j
+      acc(lc, v);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] *= p.b[j];
+      __nv_bfloat16* sT[KB];
+#pragma unroll
+      for (int i = 0; i < KB; ++i) {
+        float dd[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          float prod = 1.f;
+#pragma unroll
+          for (int l = 0; l < KB; ++l)
+            if (l != i) prod *= p.a[l][j];
+          dd[j] = v[j] * prod;
+        }
+        put_chunk(x, staging(), dd, i * e.H, cb, e.H, e.C, e.Cb);
+        sT[i] = transp();
+        put_T(x, sT[i], dd);
+        if (NS < KB) {  // one slot at a time
+          epi_sync8();
+          flush_T(x, sT[i], i * e.H + x.n0 + c0, (i + 1) * e.H);
+        }
+      }
+      if (NS >= KB) {
+        epi_sync8();
+#pragma unroll
+        for (int i = 0; i < KB; ++i) flush_T(x, sT[i], i * e.H + x.n0 + c0, (i + 1) * e.H);
+      }
+    }
+  }
+  if (MODE == TC_PLAIN && S > 1) {
+    __threadfence();
+    splitk_finish<BN, kEpiThreads>(e, x.m0, x.n0, S, tile, flag, x.et);
   }
 }
 
