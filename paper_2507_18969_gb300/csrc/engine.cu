@@ -896,6 +896,11 @@ int Model::build_tc_sites() {
     g.bn = bn;
     g.persistent = (tile_code[id] & 16) != 0;
     g.box_b = box_b;
+    g.ns = 0;
+    g.pa = a;
+    g.pb = b;
+    g.lda = a_ld;
+    g.ldb = b_ld;
     g.err = &ctl->err;
     if (precision == EDPC_FP8E4M3) {
       // e4m3 shadows of both BF16 operands, quantized before the launch
@@ -1109,6 +1114,27 @@ int Model::build_tc_sites() {
     g.ldc = F;
     EDPC_TRY(split_site(kSiteLteDownDw));
   }
+  // Over few streams the forward and dX GEMMs put the streams on the MMA's N
+  // side: the same results from a kernel with a shorter critical path. (BF16,
+  // one model; the codes of the persistent kernel are taken as they are.)
+  if (precision == EDPC_BF16 && !ngroups && !tuning_) {
+    auto few = [&](int id) -> int {
+      TcGemm& g = tcp.site[id];
+      if (g.M <= 0 || g.persistent) return EDPC_OK;
+      const int ns = tcs_streams(g.mode, g.k, g.M, g.N, g.H);
+      if (!ns) return EDPC_OK;
+      g.box_b = tcs_section_rows(g.mode, g.k);
+      EDPC_TRY(make_tmap_bf16(&g.ta, g.pb, g.N, g.K, g.ldb, g.box_b));
+      EDPC_TRY(make_tmap_bf16(&g.tb, g.pa, g.M, g.K, g.lda, ns));
+      g.ns = ns;
+      return EDPC_OK;
+    };
+    for (int kind : {BR_FWD, OUT_FWD, OUT_DX, BR_DX})
+      for (int j = 0; j < d.n; ++j) EDPC_TRY(few(blk_site(kind, j)));
+    for (int id : {kSiteHeadFwd, kSiteHeadDx}) EDPC_TRY(few(id));
+    if (d.lte)
+      for (int id : {kSiteLteDownFwd, kSiteLteUpFwd, kSiteLteUpDx, kSiteLteDownDx}) EDPC_TRY(few(id));
+  }
   // output tensor maps of every site (after its outputs and split-K factor are set)
   for (int id = 0; id < TcPlan::kMaxSites; ++id)
     if (tcp.site[id].M > 0) EDPC_TRY(tc_build_out_maps(&tcp.site[id]));
@@ -1164,6 +1190,7 @@ int Model::tune_tiles(cudaStream_t st) {
   EDPC_CUDA(cudaEventCreate(&e1));
   int r = EDPC_OK;
   const int reps = 4;
+  tuning_ = true;
   for (int id : ids) {
     float best = 1e30f;
     uint8_t best_code = 1;
@@ -1199,6 +1226,7 @@ int Model::tune_tiles(cudaStream_t st) {
     if (r != EDPC_OK) break;
     tile_code[id] = best_code;
   }
+  tuning_ = false;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (r != EDPC_OK) return r;

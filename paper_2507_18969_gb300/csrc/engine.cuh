@@ -216,6 +216,7 @@ class Model {
   void* arena_ = nullptr;
   size_t arena_bytes_ = 0;
   int nfork_ = 0;
+  bool tuning_ = false;  // the tuner times the kernels that the tile codes name
   // FP32 path
   int block_fwd(int j, const float* Xin, float* Xout, cudaStream_t st);
   int block_bwd(int j, float* dXnew, cudaStream_t st);

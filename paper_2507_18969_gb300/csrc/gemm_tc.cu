@@ -35,12 +35,13 @@ namespace {
 
 using namespace tc;
 
-// Pipeline depth: enough stages to hold the whole K panel in flight for the
-// small-N tiles (8 x 20-24 KB, one CTA per SM); 3 stages for N tiles of 96-128
-// and 2 for 192-256 (about 97 KB), so that two CTAs share an SM and one's
+// Pipeline depth. N tiles of 32 and 64: 3 and 4 stages (61 and 97 KB), so that a
+// side stream's weight gradient finds room beside a GEMM of the step (with the
+// whole K panel in flight, 8 stages, its CTAs waited for free SMs); 3 stages for
+// 96-128 and 2 for 192-256 (about 97 KB), so that two CTAs share an SM and one's
 // epilogue overlaps the other's main loop.
 template <int BN>
-constexpr int stages_for() { return BN <= 64 ? 8 : (BN <= 128 ? 3 : 2); }
+constexpr int stages_for() { return BN <= 32 ? 3 : (BN <= 64 ? 4 : (BN <= 128 ? 3 : 2)); }
 
 template <int BN>
 constexpr size_t smem_bytes() {
@@ -54,7 +55,7 @@ constexpr int kTcThreads = kEpiThreads + 64;
 // GR: grouped mode (the tile list, or each group's K range; see TcGemm). The
 // other instantiations carry none of its code.
 template <int BN, int MODE, int KB, bool F8, bool GR>
-__global__ void __launch_bounds__(kTcThreads, BN <= 64 ? 1 : 2)
+__global__ void __launch_bounds__(kTcThreads, MODE == TC_PLAIN || BN > 64 ? 2 : 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                    const __grid_constant__ CUtensorMap tmc, const __grid_constant__ CUtensorMap tmcb, const TcEpi e) {
   extern __shared__ uint8_t smem_raw[];
@@ -366,6 +367,7 @@ int tc_splitk(int M, int N, int K, int bn) {
 
 cudaError_t launch_gemm_tc(const TcGemm& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0) return cudaSuccess;
+  if (g.ns) return launch_gemm_tcs(g, st);
   if (g.fp8) {
     if (!g.inv_a || !g.inv_b) return cudaErrorInvalidValue;
     return launch_gemm_tc_t<true>(g, st);

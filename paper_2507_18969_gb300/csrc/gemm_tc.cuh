@@ -38,6 +38,12 @@ struct TcGemm {
   int splitk = 1;
   float* ws = nullptr;
   unsigned* cnt = nullptr;
+  // ns > 0: the kernel with the streams on the MMA's N side (gemm_tcs.cu), ns
+  // streams a tile. Then ta is the weights' map (box of box_b =
+  // tcs_section_rows rows) and tb the activations' (box of ns rows).
+  int ns = 0;
+  const void *pa = nullptr, *pb = nullptr;  // operands as given: A [M][K] and B [N][K], row strides
+  int lda = 0, ldb = 0;
   // Persistent kernel: one CTA per SM walks the output tiles, with two TMEM
   // accumulators so that a tile's epilogue overlaps the next tile's MMAs.
   // Same K order and epilogue arithmetic as the one-tile kernel, so the
@@ -100,6 +106,15 @@ int make_tmap_bf16_groups(CUtensorMap* tm, const void* base, uint64_t rows, uint
 cudaError_t launch_gemm_tc(const TcGemm& g, cudaStream_t st);
 // The persistent kernel (g.persistent), dispatched by launch_gemm_tc.
 cudaError_t launch_gemm_tcp(const TcGemm& g, cudaStream_t st);
+
+// The kernel for few streams (g.ns), dispatched by launch_gemm_tc.
+cudaError_t launch_gemm_tcs(const TcGemm& g, cudaStream_t st);
+// Its streams per tile (32, else 64) for M streams and N features (H hidden
+// units in the branch modes) when the tiles then fit the 152 SMs at once; else
+// 0: with more tiles than SMs the 128-row kernels re-read less.
+int tcs_streams(int mode, int k, int M, int N, int H);
+// Weight rows of a section: 128, or in the branch GEMM 128, 64, 32 for 1, 2, 3 branches.
+int tcs_section_rows(int mode, int k);
 
 // Builds g's output tensor maps (C over its logical columns: N for TC_PLAIN,
 // k * H for the branch modes; Cb likewise, H for TC_BRANCH). Returns 0 or an
