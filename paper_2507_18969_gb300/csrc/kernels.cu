@@ -1557,17 +1557,10 @@ __device__ __forceinline__ void row_cdf(const float (&p)[8], int lane, RowCdf& o
       bidx = lane * 8 + q;
     }
   }
-  const int total = warp_isum(fsum);
+  const int total = __reduce_add_sync(0xffffffffu, fsum);
   // argmax of f, lowest index on ties
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    uint32_t ob = __shfl_xor_sync(0xffffffffu, best, off);
-    int oi = __shfl_xor_sync(0xffffffffu, bidx, off);
-    if (ob > best || (ob == best && oi < bidx)) {
-      best = ob;
-      bidx = oi;
-    }
-  }
+  const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+  bidx = __reduce_min_sync(0xffffffffu, best == top ? bidx : 256);
   const int rem = kT - total;
 #pragma unroll
   for (int q = 0; q < 8; ++q)  // (constant indices keep the row in registers)
@@ -1605,14 +1598,46 @@ __device__ __forceinline__ void store_tile_T(const __nv_bfloat16* tile, int ld_s
   }
 }
 
-__global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
-  pdl_wait();
-  pdl_launch();
-  __shared__ __nv_bfloat16 tile[kRowsT][256];
+// What bounds it is one row's chain of warp reductions (the grid is a warp per
+// stream), so all that does not hang on the logits comes before the
+// dependent-launch wait: the step control, the stream's bounds, the byte to
+// encode or the decoder's state and target (all written at least two launches
+// ago), and eight rows a CTA spread 512 streams over 64 SMs. With sixteen rows
+// and everything after the wait the 64 MiB mix's step spent 8.7 us here; now
+// 4.6.
+constexpr int kRowsHead = 8;
+
+__global__ void __launch_bounds__(32 * kRowsHead) head_kernel(HeadArgs a) {
+  __shared__ __nv_bfloat16 tile[kRowsHead][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = blockIdx.x * kRowsT + warp;
+  const int s = blockIdx.x * kRowsHead + warp;
   const bool valid = s < a.b;  // warp-uniform
   const StepCtl c = *a.ctl;
+  bool active = false;
+  int x = -1;
+  DecState d{};
+  uint32_t target = 0, dr = 0;
+  if (valid) {
+    active = a.mode == 2 ? a.active[s] != 0 : (long long)c.i < a.sp.len(s);
+    if (active) {
+      if (a.mode == 0) {
+        x = a.data[a.sp.off(s) + c.i];  // warp-uniform
+      } else if (a.mode == 1) {
+        d = a.dec[s];
+        dr = d.range >> kTBits;
+        target = min(d.code / dr, (uint32_t)kT - 1);
+      } else {
+        x = a.targets[s];
+      }
+    }
+  }
+  float inv = c.inv_bact;
+  if (valid && a.rg) {  // grouped mode: the mean over the row's own group (as set_ctl / step_advance form it)
+    const int n = group_active(a.gi[a.rg[s]], c.i);
+    inv = n > 0 ? 1.0f / (float)n : 0.f;
+  }
+  pdl_wait();
+  pdl_launch();
   float dzv[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) dzv[q] = 0.f;
@@ -1636,12 +1661,6 @@ __global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) p[q] = p[q] / se;
 
-    bool active;
-    if (a.mode == 2)
-      active = a.active[s] != 0;
-    else
-      active = (long long)c.i < a.sp.len(s);
-
     RowCdf cdf;
     row_cdf(p, lane, cdf);
     if (a.freq_out) {
@@ -1653,23 +1672,12 @@ __global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
       if (lane == 31) a.cum_out[(size_t)s * 257 + 256] = (uint32_t)kT;
     }
 
-    int x = -1;
     if (active) {
       if (a.mode == 0) {
-        x = a.data[a.sp.off(s) + c.i];  // warp-uniform
         uint32_t cx = __shfl_sync(0xffffffffu, pick8(cdf.cum, x & 7), x >> 3);
         uint32_t fx = __shfl_sync(0xffffffffu, pick8(cdf.f, x & 7), x >> 3);
         if (lane == 0) a.ring[(size_t)c.slot * a.b + s] = cx | ((fx - 1u) << 16);
       } else if (a.mode == 1) {
-        DecState d;
-        uint32_t target = 0, r = 0;
-        if (lane == 0) {
-          d = a.dec[s];
-          r = d.range >> kTBits;
-          target = d.code / r;
-          if (target > (uint32_t)kT - 1) target = kT - 1;
-        }
-        target = __shfl_sync(0xffffffffu, target, 0);
         unsigned ball = __ballot_sync(0xffffffffu, cdf.cum[0] <= target);
         int L = 31 - __clz(ball);
         int cnt = 0;
@@ -1680,12 +1688,10 @@ __global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
         uint32_t cx = __shfl_sync(0xffffffffu, pick8(cdf.cum, x & 7), L);
         uint32_t fx = __shfl_sync(0xffffffffu, pick8(cdf.f, x & 7), L);
         if (lane == 0) {
-          dec_update(d, a.bits + a.bits_off[s], a.bits_len[s], r, cx, fx);
+          dec_update(d, a.bits + a.bits_off[s], a.bits_len[s], dr, cx, fx);
           a.dec[s] = d;
           a.data[a.sp.off(s) + c.i] = (uint8_t)x;
         }
-      } else {
-        x = a.targets[s];
       }
     } else if (a.mode == 0 && lane == 0) {
       a.ring[(size_t)c.slot * a.b + s] = kSkip;
@@ -1693,11 +1699,6 @@ __global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
 
     float* dz = a.dz + (size_t)s * 256 + lane * 8;
     float* po = a.p ? a.p + (size_t)s * 256 + lane * 8 : nullptr;
-    float inv = c.inv_bact;
-    if (a.rg) {  // grouped mode: the mean over the row's own group (as set_ctl / step_advance form it)
-      const int n = group_active(a.gi[a.rg[s]], c.i);
-      inv = n > 0 ? 1.0f / (float)n : 0.f;
-    }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       int j = lane * 8 + q;
@@ -1716,12 +1717,12 @@ __global__ void __launch_bounds__(32 * kRowsT) head_kernel(HeadArgs a) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) tile[warp][lane * 8 + q] = __float2bfloat16_rn(dzv[q]);
     __syncthreads();
-    store_tile_T<kRowsT>(&tile[0][0], 256, 256, blockIdx.x * kRowsT, a.dzbT, a.ldT);
+    store_tile_T<kRowsHead>(&tile[0][0], 256, 256, blockIdx.x * kRowsHead, a.dzbT, a.ldT);
   }
 }
 
 cudaError_t launch_head(const HeadArgs& a, cudaStream_t st) {
-  return launch_k(head_kernel, dim3(div_up(a.b, kRowsT)), dim3(32 * kRowsT), 0, st, a);
+  return launch_k(head_kernel, dim3(div_up(a.b, kRowsHead)), dim3(32 * kRowsHead), 0, st, a);
 }
 
 // A warp per row. What bounds it is HBM (a row is 1 KB in, 2 KB out): p and f
@@ -2108,25 +2109,53 @@ __global__ void __launch_bounds__(512) colsum_multi_kernel(ColsumJobs jobs) {
     }
   };
   if (!VEC && c < jb.cols) {
-    // rows w, w+16, ... with four interleaved accumulators
+    // rows w, w+16, ... with four interleaved accumulators; sixteen rows' loads
+    // go out together (the sums run in the same order as four at a time)
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
     int r = r_lo + w;
+    const size_t ld = (size_t)jb.ld;
+    for (; r + 240 < r_hi; r += 256) {
+      float x[16], y[16];
+      const float* px = jb.X + (size_t)r * ld + c;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) x[k] = px[(size_t)(16 * k) * ld];
+      if (jb.Y) {
+        const float* py = jb.Y + (size_t)r * ld + c;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) y[k] = py[(size_t)(16 * k) * ld];
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+          a0 = fmaf(x[k], y[k], a0);
+          a1 = fmaf(x[k + 1], y[k + 1], a1);
+          a2 = fmaf(x[k + 2], y[k + 2], a2);
+          a3 = fmaf(x[k + 3], y[k + 3], a3);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+          a0 += x[k];
+          a1 += x[k + 1];
+          a2 += x[k + 2];
+          a3 += x[k + 3];
+        }
+      }
+    }
     if (jb.Y) {
       for (; r + 48 < r_hi; r += 64) {
-        a0 += jb.X[(size_t)r * jb.ld + c] * jb.Y[(size_t)r * jb.ld + c];
-        a1 += jb.X[(size_t)(r + 16) * jb.ld + c] * jb.Y[(size_t)(r + 16) * jb.ld + c];
-        a2 += jb.X[(size_t)(r + 32) * jb.ld + c] * jb.Y[(size_t)(r + 32) * jb.ld + c];
-        a3 += jb.X[(size_t)(r + 48) * jb.ld + c] * jb.Y[(size_t)(r + 48) * jb.ld + c];
+        a0 = fmaf(jb.X[(size_t)r * ld + c], jb.Y[(size_t)r * ld + c], a0);
+        a1 = fmaf(jb.X[(size_t)(r + 16) * ld + c], jb.Y[(size_t)(r + 16) * ld + c], a1);
+        a2 = fmaf(jb.X[(size_t)(r + 32) * ld + c], jb.Y[(size_t)(r + 32) * ld + c], a2);
+        a3 = fmaf(jb.X[(size_t)(r + 48) * ld + c], jb.Y[(size_t)(r + 48) * ld + c], a3);
       }
-      for (; r < r_hi; r += 16) a0 += jb.X[(size_t)r * jb.ld + c] * jb.Y[(size_t)r * jb.ld + c];
+      for (; r < r_hi; r += 16) a0 = fmaf(jb.X[(size_t)r * ld + c], jb.Y[(size_t)r * ld + c], a0);
     } else {
       for (; r + 48 < r_hi; r += 64) {
-        a0 += jb.X[(size_t)r * jb.ld + c];
-        a1 += jb.X[(size_t)(r + 16) * jb.ld + c];
-        a2 += jb.X[(size_t)(r + 32) * jb.ld + c];
-        a3 += jb.X[(size_t)(r + 48) * jb.ld + c];
+        a0 += jb.X[(size_t)r * ld + c];
+        a1 += jb.X[(size_t)(r + 16) * ld + c];
+        a2 += jb.X[(size_t)(r + 32) * ld + c];
+        a3 += jb.X[(size_t)(r + 48) * ld + c];
       }
-      for (; r < r_hi; r += 16) a0 += jb.X[(size_t)r * jb.ld + c];
+      for (; r < r_hi; r += 16) a0 += jb.X[(size_t)r * ld + c];
     }
     a[0][0] = (a0 + a1) + (a2 + a3);
   }
