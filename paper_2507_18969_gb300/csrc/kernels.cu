@@ -948,14 +948,17 @@ cudaError_t launch_fdm_adam(const FdmSplitArgs& a, cudaStream_t st, bool persist
 // precedes the arrival counter), so the result does not depend on timing.
 // Position p = s*K + k has its D gradient values at dX[p*D ..).
 // ============================================================================================
-// Per-warp scratch of emb_range_sum: a ring of kEmbStages stages of 256 floats
-// and the list of matching positions (a 256-position block and a remainder
-// below 32).
-constexpr int kEmbStages = 4;
+// Per-warp scratch of emb_range_sum: a ring of four stages of FL floats and the
+// matching positions of one block, relative to its start.
+constexpr int kEmbBlock = 2048;  // 64 consecutive positions a lane
+template <int FL>
 struct __align__(16) EmbScratch {
-  float ring[kEmbStages][256];
-  int list[256 + 32];
+  static constexpr int kStages = 4, kFloats = FL;
+  float ring[kStages][FL];
+  uint16_t list[kEmbBlock];
 };
+using EmbDeep = EmbScratch<512>;  // two CTAs an SM: long chains, few CTAs
+using EmbWide = EmbScratch<256>;  // three CTAs an SM: many CTAs
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
@@ -970,112 +973,121 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // One warp's sum of the rows dX[p*D ..) over the positions p in [p_lo, p_hi)
 // with ctx[p] == c, in increasing p: lane d gets dimension d in a0 and d + 32 in a1.
-// What bounds it is the latency of the rows' loads when a byte value is
-// frequent (smooth images, spaces): the one warp then walks thousands of rows,
-// and the adds must stay in order. So the matches of 256 positions at a time
-// go into a list (ballots and prefix counts; the next positions' words are
-// already in flight) and their rows through a ring of asynchronous copies,
-// 1 KB a stage (256 / D rows), three stages ahead of the adds. With eight rows
-// in flight in registers instead, the 64 MiB mix's step spent 59 us here on
-// images and text; the adds' order, and so the bits, are the same.
-template <int DT>
+// The adds must stay in order, so a frequent byte's warp is bound by the
+// dependent add of its rows; all else is latency. Blocks of 2048 positions: a
+// lane compares its 64 consecutive ones at once (one load latency a block), a
+// prefix sum of the lanes' counts places their hits in the list, and the rows
+// come through a ring of asynchronous copies, up to 128 rows of 16 floats ahead
+// of the adds. Walking 256 positions at a time with ballots paid a load latency
+// each: 13.8 us for 512 streams of 32 positions (59 us with the rows loaded
+// eight at a time); now 5.7, most of it gained by loading a stage's rows into
+// registers before the serial adds (59 cycles a row as one load and add each).
+template <int DT, class Scratch>
 __device__ __forceinline__ void emb_range_sum(const uint8_t* __restrict__ ctx, const float* __restrict__ dX, int Drt,
-                                              uint32_t c, int p_lo, int p_hi, EmbScratch& s, float& a0, float& a1) {
+                                              uint32_t c, int p_lo, int p_hi, Scratch& s, float& a0, float& a1) {
+  constexpr int ST = Scratch::kStages, FL = Scratch::kFloats;
   const int lane = threadIdx.x & 31;
   const int D = DT > 0 ? DT : Drt;
-  const int R = 256 / D, C4 = D / 4, n4 = R * C4;  // rows and 16-byte pieces (at most 64) of a stage
-  const int r0 = lane / C4, q0 = (lane - r0 * C4) * 4;
-  const int r1 = (lane + 32) / C4, q1 = (lane + 32 - r1 * C4) * 4;
-  const bool al4 = (reinterpret_cast<uintptr_t>(ctx) & 3) == 0 && (p_lo & 3) == 0;
+  const int R = FL / D, C4 = D / 4;  // rows of a stage, 16-byte pieces of a row
+  const int l0 = min(lane, D - 1), l1 = min(lane + 32, D - 1);
+  const uint32_t cc = c * 0x01010101u;
   a0 = a1 = 0.f;
-  int pend = 0, issued = 0, consumed = 0;
-  auto issue = [&](int first, int n) {
-    float* st = s.ring[issued % kEmbStages];
-    if (r0 < n && lane < n4) cp_async16(st + r0 * D + q0, dX + (size_t)s.list[first + r0] * D + q0);
-    if (r1 < n && lane + 32 < n4) cp_async16(st + r1 * D + q1, dX + (size_t)s.list[first + r1] * D + q1);
-    cp_async_commit();
-    ++issued;
-  };
-  auto add = [&](int n) {
-    const float* st = s.ring[consumed % kEmbStages];
+  for (int pb = p_lo; pb < p_hi; pb += kEmbBlock) {
+    // hits of positions [q0, q0 + 64): bit k of m is q0 + k
+    const int q0 = pb + lane * 64;
+    unsigned long long m = 0;
 #pragma unroll
-    for (int r = 0; r < (DT > 0 ? 256 / (DT > 0 ? DT : 1) : n); ++r) {
-      if (r >= n) break;
-      if (lane < D) a0 += st[r * D + lane];
-      if (lane + 32 < D) a1 += st[r * D + lane + 32];
-    }
-    ++consumed;
-  };
-  auto word = [&](int pw) -> uint32_t {  // positions pw..pw+3 (a non-matching byte past p_hi)
-    if (al4 && pw + 4 <= p_hi) return *reinterpret_cast<const uint32_t*>(ctx + pw);
-    uint32_t x = 0;
-    for (int u = 0; u < 4; ++u) x |= (uint32_t)(pw + u < p_hi ? ctx[pw + u] : (uint8_t)(c ^ 1u)) << (8 * u);
-    return x;
-  };
-  const uint32_t below = (1u << lane) - 1u;
-  uint32_t nx[2];
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + 16 * u;
+      uint32_t w[4];
+      if (q + 16 <= p_hi && ((reinterpret_cast<uintptr_t>(ctx) + q) & 15) == 0) {
+        const uint4 x = *reinterpret_cast<const uint4*>(ctx + q);
+        w[0] = x.x;
+        w[1] = x.y;
+        w[2] = x.z;
+        w[3] = x.w;
+      } else {
 #pragma unroll
-  for (int k = 0; k < 2; ++k) nx[k] = word(p_lo + k * 128 + 4 * lane);
-  for (int pb = p_lo; pb < p_hi; pb += 256) {
-    const uint32_t xs[2] = {nx[0], nx[1]};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) nx[k] = word(pb + 256 + k * 128 + 4 * lane);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      uint32_t at = (uint32_t)pend;
-      bool hit[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        hit[u] = ((xs[k] >> (8 * u)) & 0xffu) == c;
-        const uint32_t m = __ballot_sync(0xffffffffu, hit[u]);
-        at += __popc(m & below);
-        pend += __popc(m);
+        for (int k = 0; k < 4; ++k) {
+          w[k] = ~cc;  // never matches
+          for (int t = 0; t < 4; ++t)
+            if (q + 4 * k + t < p_hi) w[k] = (w[k] & ~(0xFFu << (8 * t))) | (uint32_t)ctx[q + 4 * k + t] << (8 * t);
+        }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (hit[u]) s.list[at++] = pb + k * 128 + 4 * lane + u;
+      for (int k = 0; k < 4; ++k) {
+        // 0xFF bytes where equal -> one bit each, in byte order
+        const uint32_t eq = __vcmpeq4(w[k], cc) & 0x08040201u;
+        m |= (unsigned long long)((eq | eq >> 8 | eq >> 16 | eq >> 24) & 15u) << (16 * u + 4 * k);
+      }
+    }
+    const int cnt = __popcll(m);
+    int at = cnt;  // inclusive prefix sum over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += v;
+    }
+    const int n = __shfl_sync(0xffffffffu, at, 31);
+    if (n == 0) continue;  // warp-uniform
+    at -= cnt;
+    while (m) {
+      s.list[at++] = (uint16_t)(lane * 64 + __ffsll((long long)m) - 1);
+      m &= m - 1;
     }
     __syncwarp();
-    int done = 0;
-    for (; pend - done >= R; done += R) {  // warp-uniform
-      if (issued - consumed == kEmbStages) {
-        cp_async_wait<kEmbStages - 1>();
-        __syncwarp();
-        add(R);
-        __syncwarp();
+    const float* rows = dX + (size_t)pb * D;
+    const int stages = (n + R - 1) / R;
+    auto issue = [&](int k) {
+      if (k < stages) {
+        float* st = s.ring[k % ST];
+        const int r_n = min(R, n - k * R);
+#pragma unroll
+        for (int u = 0; u < FL / 128; ++u) {
+          const int r = (lane + 32 * u) / C4, q = (lane + 32 * u - r * C4) * 4;
+          if (r < r_n) cp_async16(st + r * D + q, rows + (size_t)s.list[k * R + r] * D + q);
+        }
       }
-      issue(done, R);
-    }
-    if (done) {
-      pend -= done;
-      const int v = lane < pend ? s.list[done + lane] : 0;
+      cp_async_commit();
+    };
+    for (int k = 0; k < ST; ++k) issue(k);
+    for (int k = 0; k < stages; ++k) {
+      cp_async_wait<ST - 1>();
       __syncwarp();
-      if (lane < pend) s.list[lane] = v;
+      const float* st = s.ring[k % ST];
+      const int r_n = min(R, n - k * R);
+      // (lanes beyond D add some other dimension's values, which nothing reads)
+      if (DT > 0 && DT <= 32 && r_n == R) {
+        constexpr int RR = DT > 0 ? FL / (DT > 0 ? DT : 1) : 1;
+        float v[RR];  // the loads first: only the adds are serial
+#pragma unroll
+        for (int r = 0; r < RR; ++r) v[r] = st[r * D + l0];
+#pragma unroll
+        for (int r = 0; r < RR; ++r) a0 += v[r];
+      } else {
+#pragma unroll 4
+        for (int r = 0; r < r_n; ++r) {
+          a0 += st[r * D + l0];
+          if (D > 32) a1 += st[r * D + l1];
+        }
+      }
+      __syncwarp();  // the stage is read before its next copies
+      issue(k + ST);
     }
-    __syncwarp();
-  }
-  while (issued > consumed) {
     cp_async_wait<0>();
     __syncwarp();
-    add(R);
-  }
-  if (pend) {
-    __syncwarp();
-    issue(0, pend);
-    cp_async_wait<0>();
-    __syncwarp();
-    add(pend);
   }
 }
 
-template <int DT>
+template <int DT, class Scratch>
 __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __restrict__ ctx,
                                                               const float* __restrict__ dX, int P, int D,
                                                               float* __restrict__ dE, float* __restrict__ part,
                                                               unsigned* __restrict__ cnt) {
   pdl_wait();
   pdl_launch();
-  __shared__ EmbScratch scratch[8];
+  extern __shared__ __align__(16) unsigned char emb_smem[];
+  Scratch* scratch = reinterpret_cast<Scratch*>(emb_smem);
   __shared__ float wsum[8][64];
   __shared__ int is_last;
   const uint32_t c = blockIdx.x;
@@ -1119,6 +1131,26 @@ __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __r
 
 int embed_bwd_chunks(int b, int K) { return (b * K + kEmbChunkPos - 1) / kEmbChunkPos; }
 
+template <int DT, class Scratch, class... A>
+static cudaError_t launch_emb_owner(dim3 grid, cudaStream_t st, A... args) {
+  constexpr size_t smem = 8 * sizeof(Scratch);
+  auto k = embed_bwd_owner_kernel<DT, Scratch>;
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once,
+                 [&] { attr = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+  if (attr != cudaSuccess) return attr;
+  return launch_k(k, grid, dim3(256), smem, st, args...);
+}
+
+template <int DT>
+static cudaError_t launch_emb(dim3 grid, cudaStream_t st, const uint8_t* ctx, const float* dX, int P, int D, float* dE,
+                              float* part, unsigned* cnt) {
+  // 256 CTAs (one chunk) are resident at once with the deep ring; with several chunks more CTAs an SM count more
+  if (grid.y == 1) return launch_emb_owner<DT, EmbDeep>(grid, st, ctx, dX, P, D, dE, part, cnt);
+  return launch_emb_owner<DT, EmbWide>(grid, st, ctx, dX, P, D, dE, part, cnt);
+}
+
 cudaError_t launch_embed_bwd(const uint8_t* ctx, const float* dX, int b, int K, int D, float* dE, float* part,
                              unsigned* cnt, cudaStream_t st) {
   if (D > 64) return cudaErrorInvalidValue;
@@ -1126,9 +1158,9 @@ cudaError_t launch_embed_bwd(const uint8_t* ctx, const float* dX, int b, int K, 
   if (nq > 1 && (!part || !cnt)) return cudaErrorInvalidValue;
   const dim3 grid(256, nq < 1 ? 1 : nq);
   switch (D) {  // the configurations' widths have their loops unrolled
-    case 8: return launch_k(embed_bwd_owner_kernel<8>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
-    case 16: return launch_k(embed_bwd_owner_kernel<16>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
-    default: return launch_k(embed_bwd_owner_kernel<0>, grid, dim3(256), 0, st, ctx, dX, b * K, D, dE, part, cnt);
+    case 8: return launch_emb<8>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
+    case 16: return launch_emb<16>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
+    default: return launch_emb<0>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
   }
 }
 
@@ -1144,7 +1176,8 @@ __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __
                                                                const GroupInfo* __restrict__ gi, size_t gs) {
   pdl_wait();
   pdl_launch();
-  __shared__ EmbScratch scratch[8];
+  extern __shared__ __align__(16) unsigned char emb_smem[];
+  EmbWide* scratch = reinterpret_cast<EmbWide*>(emb_smem);
   __shared__ float part[8][64];
   const GroupInfo g = gi[blockIdx.x];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1160,11 +1193,22 @@ __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __
   part[w][lane + 32] = a1;
   __syncthreads();
   if ((w & 3) == 0) {
-    float* out = dE + (size_t)blockIdx.x * gs + (size_t)c * D;
-    if (lane < D) out[lane] = ((part[w][lane] + part[w + 1][lane]) + part[w + 2][lane]) + part[w + 3][lane];
-    if (lane + 32 < D)
-      out[lane + 32] = ((part[w][lane + 32] + part[w + 1][lane + 32]) + part[w + 2][lane + 32]) + part[w + 3][lane + 32];
+    const size_t o = (size_t)blockIdx.x * gs + (size_t)c * D;
+    for (int d = lane; d < D; d += 32)
+      dE[o + d] = ((part[w][d] + part[w + 1][d]) + part[w + 2][d]) + part[w + 3][d];
   }
+}
+
+template <int DT, class... A>
+static cudaError_t launch_emb_groups(dim3 grid, cudaStream_t st, A... args) {
+  constexpr size_t smem = 8 * sizeof(EmbWide);
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(embed_bwd_groups_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  });
+  if (attr != cudaSuccess) return attr;
+  return launch_k(embed_bwd_groups_kernel<DT>, grid, dim3(256), smem, st, args...);
 }
 
 cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, int D, float* dE,
@@ -1173,9 +1217,9 @@ cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, 
     return cudaErrorInvalidValue;
   const dim3 grid(ngroups, 128);
   switch (D) {
-    case 8: return launch_k(embed_bwd_groups_kernel<8>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
-    case 16: return launch_k(embed_bwd_groups_kernel<16>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
-    default: return launch_k(embed_bwd_groups_kernel<0>, grid, dim3(256), 0, st, ctx, dX, K, D, dE, gi, gs);
+    case 8: return launch_emb_groups<8>(grid, st, ctx, dX, K, D, dE, gi, gs);
+    case 16: return launch_emb_groups<16>(grid, st, ctx, dX, K, D, dE, gi, gs);
+    default: return launch_emb_groups<0>(grid, st, ctx, dX, K, D, dE, gi, gs);
   }
 }
 
