@@ -59,7 +59,9 @@ struct StepCtl {
   float lr;
   int err;        // sticky error bits
   int cpi;        // next entry of the active-count table (uneven splits)
-  int pad[6];
+  float a_lr, a_bc1, a_bc2;  // lr, bc1 and bc2 as Adam reads them: set by the head kernel, so that the record
+                             // can be advanced before the step's Adam has run
+  int pad[3];
 };
 
 // Change point of the active-stream count: from time index i on, bact

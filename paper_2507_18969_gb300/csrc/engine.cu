@@ -11,8 +11,7 @@
 //   adjoint is fused with the FDM's Adam update. Adam on the shared params.
 //
 // Two arithmetic paths share this sequence:
-//   FP32  SIMT GEMMs and separate element-wise kernels; weight gradients and
-//         column sums on the side stream as below.
+//   FP32  SIMT GEMMs and separate element-wise kernels.
 //   BF16  tcgen05 GEMMs whose epilogues fuse the MBRB element-wise ops and
 //         write the BF16 (and transposed BF16) operands of the next GEMMs; the
 //         weight-gradient GEMMs and column sums, which nothing on the step's
@@ -121,6 +120,9 @@ __global__ void set_ctl_kernel(StepCtl* ctl, int i, int t, int bact, int slot, f
   c.bc2 = 1.0f - powf(kB2, (float)t);
   c.slot = slot;
   c.lr = lr;
+  c.a_lr = lr;
+  c.a_bc1 = c.bc1;
+  c.a_bc2 = c.bc2;
   c.err = 0;
   *ctl = c;
 }
@@ -132,14 +134,13 @@ Model::~Model() {
     if (e) cudaEventDestroy(e);
   for (auto& e : fork)
     if (e) cudaEventDestroy(e);
-  if (join_ev) cudaEventDestroy(join_ev);
   if (tr_ev) cudaEventDestroy(tr_ev);
-  if (fdm_join_ev) cudaEventDestroy(fdm_join_ev);
   if (dx_ev) cudaEventDestroy(dx_ev);
   if (adam_ev) cudaEventDestroy(adam_ev);
   if (tick_ev) cudaEventDestroy(tick_ev);
   if (bwd_ev) cudaEventDestroy(bwd_ev);
   if (side) cudaStreamDestroy(side);
+  if (side2) cudaStreamDestroy(side2);
   if (side_fdm) cudaStreamDestroy(side_fdm);
   if (bwd_st) cudaStreamDestroy(bwd_st);
   if (gU) cudaFree(gU);
@@ -189,14 +190,18 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
         for (int c0 = 0; c0 < cols; c0 += 32) th.push_back({off, rows, cols, r0, c0});
     };
     for (int j = 0; j < d.n; ++j) {
+      tile_lo[j] = (int)th.size();
       mat(po.blk[j].W, kH, d.F);
       mat(po.blk[j].Wo, d.F, d.H);
     }
+    tile_lo[d.n] = (int)th.size();
     if (d.lte) {
       mat(po.W1, d.Fp, d.F);
       mat(po.W2, d.F, d.Fp);
     }
+    tile_lo[d.n + 1] = (int)th.size();
     mat(po.Wh, 256, d.F);
+    tile_lo[d.n + 2] = (int)th.size();
     if (ngroups > 1) {  // every group's matrices
       const size_t n1 = th.size();
       for (int g = 1; g < ngroups; ++g)
@@ -439,10 +444,8 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
     EDPC_TRY(build_tc_plan());
     EDPC_CUDA(cudaEventCreateWithFlags(&tr_ev, cudaEventDisableTiming));
   }
-  EDPC_CUDA(cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, delayed ? prio_greatest : prio_least));
+  for (auto* q : {&side, &side2}) EDPC_CUDA(cudaStreamCreateWithPriority(q, cudaStreamNonBlocking, prio_greatest));
   for (auto& e : fork) EDPC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  EDPC_CUDA(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
-  EDPC_CUDA(cudaEventCreateWithFlags(&fdm_join_ev, cudaEventDisableTiming));
   if (split) {
     EDPC_CUDA(cudaStreamCreateWithPriority(&side_fdm, cudaStreamNonBlocking, prio_least));
     EDPC_CUDA(cudaEventCreateWithFlags(&dx_ev, cudaEventDisableTiming));
@@ -609,7 +612,10 @@ int Model::fdm_fwd_call(const StepIO& io, cudaStream_t st) {
 }
 
 int Model::forward_f32(const StepIO& io, cudaStream_t st) {
-  EDPC_CUDA(launch_embed(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx, st));
+  {
+    PdlScope scope(delayed);  // else: follows the join of the side streams
+    EDPC_CUDA(launch_embed(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx, st));
+  }
   for (int j = 0; j < d.nloc; ++j) EDPC_TRY(block_fwd(j, S[j], S[j + 1], st));
   if (d.lte) EDPC_TRY(linear_fwd(S[d.nloc], d.b, d.F, po.W1, po.b1, d.Fp, nullptr, Xp, st));  // Eq. 14
   EDPC_TRY(fdm_fwd_call(io, st));  // Eq. 15 (w/o LTE: on S[nloc] into S[nloc + 1])
@@ -620,17 +626,23 @@ int Model::forward_f32(const StepIO& io, cudaStream_t st) {
 }
 
 // The weight gradients and column sums of a layer, which nothing on the step's
-// critical path waits for, run on the side stream; so every gradient they read
+// critical path waits for, run on the side streams; so every gradient they read
 // has a buffer of its own per block.
 int Model::side_f32(const float* dOut, int out, const float* X, int in, size_t w_off, ColsumJobs cj, cudaStream_t st) {
-  EDPC_TRY(fork_side(st));
-  NoPdl scope;
-  if (X) EDPC_TRY(linear_dw(dOut, d.b, out, X, in, w_off, side));
-  if (cj.n) EDPC_CUDA(launch_colsum(cj, side));
+  if (X) {
+    EDPC_TRY(fork_to(st, side));
+    NoPdl scope;
+    EDPC_TRY(linear_dw(dOut, d.b, out, X, in, w_off, side));
+  }
+  if (cj.n) {
+    EDPC_TRY(fork_to(st, side2));
+    NoPdl scope;
+    EDPC_CUDA(launch_colsum(cj, side2));
+  }
   return EDPC_OK;
 }
 
-int Model::block_bwd(int j, float* dXnew, cudaStream_t st) {
+int Model::block_bwd(const StepIO& io, int j, float* dXnew, cudaStream_t st) {
   const BlockOff& o = po.blk[j];
   BlockAct& a = ba[j];
   BlockBf16& q = bb[j];
@@ -652,7 +664,7 @@ int Model::block_bwd(int j, float* dXnew, cudaStream_t st) {
   EDPC_TRY(side_f32(nullptr, 0, nullptr, 0, 0, cj, st));
   // Eq. 9: X0 = g * xhat + beta, plus the residual path of Eq. 13
   EDPC_CUDA(launch_ln_bwd(q.dX0, a.xhat, a.rstd, P + o.ln_g, q.dOut, dXnew, d.b, d.F, st));
-  return EDPC_OK;
+  return adam_layer(io, j, st);
 }
 
 int Model::flush(cudaStream_t st) {
@@ -737,6 +749,7 @@ int Model::backward_f32(const StepIO& io, cudaStream_t st) {
   };
   EDPC_TRY(side_f32(dz, 256, S[d.n + 1], d.F, po.Wh, one(dz, 256, po.bh), st));
   EDPC_TRY(linear_dx(dz, d.b, 256, po.Wh, d.F, bb[d.n - 1].dOut, st));
+  EDPC_TRY(adam_layer(io, d.n + 1, st));
   auto middle = [&]() -> int {  // between the Global and the Local blocks
     if (!d.lte) return fdm_bwd_joined(io, st);  // the FDM's adjoint alone: dLte -> dXp
     // LTE up (Eq. 16)
@@ -746,18 +759,16 @@ int Model::backward_f32(const StepIO& io, cudaStream_t st) {
     EDPC_TRY(fdm_bwd_joined(io, st));
     // LTE down (Eq. 14)
     EDPC_TRY(side_f32(dXp, d.Fp, S[d.nloc], d.F, po.W1, one(dXp, d.Fp, po.b1), st));
-    return linear_dx(dXp, d.b, d.Fp, po.W1, d.F, d.nloc > 0 ? bb[d.nloc - 1].dOut : dh0, st);
+    EDPC_TRY(linear_dx(dXp, d.b, d.Fp, po.W1, d.F, d.nloc > 0 ? bb[d.nloc - 1].dOut : dh0, st));
+    return adam_layer(io, d.n, st);
   };
   for (int j = d.n - 1; j >= 0; --j) {
     if (j == d.nloc - 1) EDPC_TRY(middle());
-    EDPC_TRY(block_bwd(j, j == d.nloc ? dLte : (j == 0 ? dh0 : bb[j - 1].dOut), st));
+    EDPC_TRY(block_bwd(io, j, j == d.nloc ? dLte : (j == 0 ? dh0 : bb[j - 1].dOut), st));
   }
   if (d.nloc == 0) EDPC_TRY(middle());
-  EDPC_CUDA(launch_embed_bwd(ctx, dh0, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, st));
-  // join the side stream
-  EDPC_CUDA(cudaEventRecord(join_ev, side));
-  EDPC_CUDA(cudaStreamWaitEvent(st, join_ev, 0));
-  return EDPC_OK;
+  EDPC_CUDA(launch_embed_bwd(ctx, dh0, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, advance_of(io), emb_adam(io), st));
+  return join_sides(st);
 }
 
 // ==========================================================================================
@@ -1309,41 +1320,111 @@ int Model::colsums(ColsumJobs cj, cudaStream_t st) {
   return EDPC_OK;
 }
 
-int Model::fork_side(cudaStream_t st) {
+// `to` waits for everything launched so far on `from`.
+int Model::fork_to(cudaStream_t from, cudaStream_t to) {
   if (nfork_ >= kForks) return fail(EDPC_EINVAL, "too many side-stream forks in one step");
   cudaEvent_t e = fork[nfork_++];
-  EDPC_CUDA(cudaEventRecord(e, st));
-  EDPC_CUDA(cudaStreamWaitEvent(side, e, 0));
+  EDPC_CUDA(cudaEventRecord(e, from));
+  EDPC_CUDA(cudaStreamWaitEvent(to, e, 0));
   return EDPC_OK;
 }
 
+int Model::fork_side(cudaStream_t st) { return fork_to(st, side); }
+
+int Model::join_sides(cudaStream_t st) {
+  EDPC_TRY(fork_to(side, st));
+  return fork_to(side2, st);
+}
+
+// Adam of a layer (block j, d.n: the LTE, d.n + 1: the head) on the second side
+// stream, once its gradients are complete there and on the first one, and the
+// adjoint on st no longer reads its weights.
+int Model::adam_layer(const StepIO& io, int layer, cudaStream_t st) {
+  if (!io.update || delayed || (layer == d.n && !d.lte)) return EDPC_OK;
+  EDPC_TRY(fork_to(st, side2));
+  EDPC_TRY(fork_to(side, side2));
+  AdamLayer a;
+  a.P = P;
+  a.M = M;
+  a.V = V;
+  a.G = G;
+  a.ctl = ctl;
+  auto vec = [&](size_t off, size_t n) { a.vec[a.nvec++] = {off, n}; };
+  const size_t end = layer < d.n - 1 ? po.blk[layer + 1].ln_g : (layer == d.n - 1 ? (d.lte ? po.W1 : po.Wh)
+                     : (layer == d.n ? po.Wh : po.total));
+  if (precision == EDPC_FP32) {
+    const size_t lo = layer < d.n ? po.blk[layer].ln_g : (layer == d.n ? po.W1 : po.Wh);
+    vec(lo, end - lo);
+  } else {
+    a.Pb = Pb;
+    a.PbT = PbT;
+    a.tiles = tiles + tile_lo[layer];
+    a.ntiles = tile_lo[layer + 1] - tile_lo[layer];
+    if (layer < d.n) {
+      const BlockOff& o = po.blk[layer];
+      vec(o.ln_g, o.W - o.ln_g);
+      vec(o.c, o.Wo - o.c);
+      vec(o.co, end - o.co);
+    } else if (layer == d.n) {
+      vec(po.b1, po.W2 - po.b1);
+      vec(po.b2, end - po.b2);
+    } else {
+      vec(po.bh, end - po.bh);
+    }
+  }
+  if (ngroups) {
+    a.groups = (unsigned)ngroups;
+    a.gs = gstride;
+  }
+  NoPdl scope;
+  EDPC_CUDA(launch_adam_layer(a, side2));
+  return EDPC_OK;
+}
+
+// The embedding table's Adam, in the launch that forms its gradient.
+EmbAdam Model::emb_adam(const StepIO& io) const {
+  EmbAdam u;
+  if (io.update && !delayed) {
+    u.P = P + po.E;
+    u.M = M + po.E;
+    u.V = V + po.E;
+    u.Pb = Pb ? Pb + po.E : nullptr;
+    u.ctl = ctl;
+  }
+  return u;
+}
+
 int Model::forward_bf16(const StepIO& io, cudaStream_t st) {
-  nfork_ = 0;
   const bool f8m = precision == EDPC_FP8E4M3;
   if (f8m) {
     std::fill(f8_done.begin(), f8_done.end(), 0);
+    NoPdl scope;  // follows the join of the side streams
     EDPC_CUDA(launch_zero_u32(f8_amax, (int)f8.size(), st));  // this step's amax slots
   }
-  // Transposed BF16 weight copies for this step's dX GEMMs, from the weights the
-  // previous Adam wrote, on the side stream while the forward pass runs.
-  EDPC_TRY(fork_side(st));
-  {
+  if (delayed || f8m) {
+    // Delayed update: transposed BF16 weight copies for the adjoint, from the
+    // weights the previous Adam wrote, on the side stream while the forward
+    // pass runs (otherwise Adam writes them). FP8: the transposed shadows.
+    EDPC_TRY(fork_to(st, side));
     NoPdl scope;
-    EDPC_CUDA(launch_transpose_tiles(Pb, PbT, tiles, ntiles, side));
+    if (delayed) EDPC_CUDA(launch_transpose_tiles(Pb, PbT, tiles, ntiles, side));
     if (f8m) EDPC_TRY(quantize_weights(true, side));
+    EDPC_CUDA(cudaEventRecord(tr_ev, side));
   }
-  EDPC_CUDA(cudaEventRecord(tr_ev, side));
   if (f8m) EDPC_TRY(quantize_weights(false, st));
   // the embedding, fused with the first block's LayerNorm when a Local block follows it
   const bool fuse0 = d.nloc > 0 && (d.F == 128 || d.F == 256 || d.F == 512 || d.F == 1024);
-  if (fuse0) {
-    const BlockOff& o = po.blk[0];
-    EDPC_CUDA(launch_embed_ln_bf16(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx,
-                                   P + o.ln_g, P + o.ln_b, ba[0].xhat, ba[0].rstd, bb[0].X0b, bb[0].X0bT, d.ldT, st,
-                                   row_grp, gstride));  // Eq. 9 of block 0
-  } else {
-    EDPC_CUDA(launch_embed(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx, st,
-                           row_grp, gstride));
+  {
+    PdlScope scope(delayed || f8m);  // else: follows the join of the side streams
+    if (fuse0) {
+      const BlockOff& o = po.blk[0];
+      EDPC_CUDA(launch_embed_ln_bf16(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx,
+                                     P + o.ln_g, P + o.ln_b, ba[0].xhat, ba[0].rstd, bb[0].X0b, bb[0].X0bT, d.ldT, st,
+                                     row_grp, gstride));  // Eq. 9 of block 0
+    } else {
+      EDPC_CUDA(launch_embed(io.mode == 2 ? nullptr : io.data, io.sp, ctl, P + po.E, d.b, d.K, d.D, S[0], ctx, st,
+                             row_grp, gstride));
+    }
   }
   if (d.nloc == 0) EDPC_CUDA(launch_to_bf16(S[0], d.b, d.F, d.F, Slte_b, d.F, Slte_bT, d.ldT, st));
   for (int jj = 0; jj < d.n; ++jj) {
@@ -1370,17 +1451,17 @@ int Model::fdm_bwd_joined(const StepIO& io, cudaStream_t st) {
   // streaming) runs faster alone than beside the side stream's pending
   // weight gradients, so it waits for them (measured: 6.63 -> 5.81 ms per
   // step at 4096 streams; at 512 streams the overlap wins).
-  EDPC_CUDA(cudaEventRecord(fdm_join_ev, side));
-  EDPC_CUDA(cudaStreamWaitEvent(st, fdm_join_ev, 0));
-  NoPdl scope;  // two incoming dependencies
+  EDPC_TRY(join_sides(st));
+  NoPdl scope;  // several incoming dependencies
   return fdm_bwd_call(io, st);
 }
 
 int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
   const int kH = d.k * d.H;
-  // PbT is read by the dX GEMMs below (delayed update: this parity's copies
-  // were made during the previous step)
-  if (!delayed) EDPC_CUDA(cudaStreamWaitEvent(st, tr_ev, 0));
+  nfork_ = 0;  // (FP8's fork in the forward pass has its event waited for by then)
+  const bool f8m = precision == EDPC_FP8E4M3;
+  // the dX GEMMs read FP8's transposed shadows (delayed update: made during the previous step)
+  if (f8m && !delayed) EDPC_CUDA(cudaStreamWaitEvent(st, tr_ev, 0));
   // side: head weight gradients
   EDPC_TRY(fork_side(st));
   EDPC_TRY(run_tc(kSiteHeadDw, side));
@@ -1388,12 +1469,14 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     ColsumJobs cj{};
     cj.job[0] = {dz, nullptr, d.b, 256, 256, G + po.bh};
     cj.n = 1;
-    EDPC_TRY(colsums(cj, side));
+    EDPC_TRY(fork_to(st, side2));
+    EDPC_TRY(colsums(cj, side2));
   }
   {
-    NoPdl scope;  // the stream also waits on the transposes' event
+    PdlScope scope(!f8m);  // FP8: the stream also waits on the shadows' event
     EDPC_TRY(run_tc(kSiteHeadDx, st));  // dOut of the last block
   }
+  EDPC_TRY(adam_layer(io, d.n + 1, st));
   for (int j = d.n - 1; j >= 0; --j) {
     const BlockOff& o = po.blk[j];
     BlockBf16& q = bb[j];
@@ -1405,7 +1488,8 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
       ColsumJobs cj{};
       cj.job[0] = {dLte, nullptr, d.b, d.F, d.F, G + po.b2};
       cj.n = 1;
-      EDPC_TRY(colsums(cj, side));
+      EDPC_TRY(fork_to(st, side2));
+      EDPC_TRY(colsums(cj, side2));
       EDPC_TRY(run_tc(kSiteLteUpDx, st));
       EDPC_TRY(fdm_bwd_joined(io, st));
       EDPC_TRY(fork_side(st));
@@ -1413,8 +1497,10 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
       ColsumJobs cj2{};
       cj2.job[0] = {dXp, nullptr, d.b, d.Fp, d.Fp, G + po.b1};
       cj2.n = 1;
-      EDPC_TRY(colsums(cj2, side));
+      EDPC_TRY(fork_to(st, side2));
+      EDPC_TRY(colsums(cj2, side2));
       EDPC_TRY(run_tc(kSiteLteDownDx, st));
+      EDPC_TRY(adam_layer(io, d.n, st));
     }
     EDPC_TRY(fork_side(st));  // dOut_j is ready
     EDPC_TRY(run_tc(blk_site(OUT_DW, j), side));
@@ -1422,7 +1508,7 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     EDPC_TRY(fork_side(st));
     EDPC_TRY(run_tc(blk_site(BR_DW, j), side));
     EDPC_TRY(run_tc(blk_site(BR_DX, j), st));  // dX0 (adjoint of Eq. 10)
-    EDPC_TRY(fork_side(st));
+    EDPC_TRY(fork_to(st, side2));
     {
       ColsumJobs cj{};
       cj.job[0] = {q.dOut, nullptr, d.b, d.F, d.F, G + o.co};
@@ -1430,7 +1516,7 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
       cj.job[2] = {q.dX0, ba[j].xhat, d.b, d.F, d.F, G + o.ln_g};
       cj.job[3] = {q.dX0, nullptr, d.b, d.F, d.F, G + o.ln_b};
       cj.n = 4;
-      EDPC_TRY(colsums(cj, side));
+      EDPC_TRY(colsums(cj, side2));
     }
     // LN adjoint (Eq. 9) + residual path: gradient of the block input
     float* out;
@@ -1448,6 +1534,7 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     }
     EDPC_CUDA(launch_ln_bwd_bf16(q.dX0, ba[j].xhat, ba[j].rstd, P + o.ln_g, q.dOut, out, outb, outbT, d.b, d.F,
                                  d.ldT, st, row_grp, gstride));
+    EDPC_TRY(adam_layer(io, j, st));
   }
   if (d.nloc == 0 && !d.lte) EDPC_TRY(fdm_bwd_joined(io, st));  // w/o LTE: writes dh0
   if (d.nloc == 0 && d.lte) {
@@ -1457,7 +1544,8 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     ColsumJobs cj{};
     cj.job[0] = {dLte, nullptr, d.b, d.F, d.F, G + po.b2};
     cj.n = 1;
-    EDPC_TRY(colsums(cj, side));
+    EDPC_TRY(fork_to(st, side2));
+    EDPC_TRY(colsums(cj, side2));
     EDPC_TRY(run_tc(kSiteLteUpDx, st));
     EDPC_TRY(fdm_bwd_call(io, st));
     EDPC_TRY(fork_side(st));
@@ -1465,17 +1553,17 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     ColsumJobs cj2{};
     cj2.job[0] = {dXp, nullptr, d.b, d.Fp, d.Fp, G + po.b1};
     cj2.n = 1;
-    EDPC_TRY(colsums(cj2, side));
+    EDPC_TRY(fork_to(st, side2));
+    EDPC_TRY(colsums(cj2, side2));
     EDPC_TRY(run_tc(kSiteLteDownDx, st));  // writes dh0
+    EDPC_TRY(adam_layer(io, d.n, st));
   }
   if (ngroups)
-    EDPC_CUDA(launch_embed_bwd_groups(ctx, dh0, d.K, d.D, G + po.E, ginfo, ngroups, gstride, st));
+    EDPC_CUDA(launch_embed_bwd_groups(ctx, dh0, d.K, d.D, G + po.E, ginfo, ngroups, gstride, advance_of(io),
+                                      emb_adam(io), st));
   else
-    EDPC_CUDA(launch_embed_bwd(ctx, dh0, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, st));
-  // join the side stream
-  EDPC_CUDA(cudaEventRecord(join_ev, side));
-  EDPC_CUDA(cudaStreamWaitEvent(st, join_ev, 0));
-  return EDPC_OK;
+    EDPC_CUDA(launch_embed_bwd(ctx, dh0, d.b, d.K, d.D, G + po.E, emb_part, emb_cnt, advance_of(io), emb_adam(io), st));
+  return join_sides(st);
 }
 
 // ==========================================================================================
@@ -1516,15 +1604,18 @@ int Model::backward(const StepIO& io, cudaStream_t st) {
   return precision != EDPC_FP32 ? backward_bf16(io, st) : backward_f32(io, st);
 }
 
-int Model::adam(cudaStream_t st) {
-  if (precision != EDPC_FP32) {
-    NoPdl scope;  // follows the join of the side stream
-    EDPC_CUDA(launch_adam_bf16(P, G, M, V, Pb, np_all, ctl, st));
-  } else {
-    NoPdl scope;
-    EDPC_CUDA(launch_adam(P, G, M, V, nparam, ctl, st));
+// The embedding adjoint, the last launch on the step's stream, advances the step
+// control (the delayed update has two records, advanced by a launch of its own).
+Advance Model::advance_of(const StepIO& io) const {
+  Advance a;
+  if (io.advance && !delayed) {
+    a.ctl = ctl;
+    a.sp = io.sp;
+    a.K = d.K;
+    a.ring_slots = io.ring_slots;
+    a.b = d.b;
   }
-  return EDPC_OK;
+  return a;
 }
 
 int Model::step(const StepIO& io, cudaStream_t st) {
@@ -1532,9 +1623,7 @@ int Model::step(const StepIO& io, cudaStream_t st) {
   EDPC_TRY(forward(io, st));
   EDPC_TRY(head(io, st));
   EDPC_TRY(backward(io, st));
-  if (io.update) EDPC_TRY(adam(st));
-  if (io.advance) EDPC_CUDA(launch_step_advance(ctl, io.sp, d.K, io.ring_slots, d.b, st));
-  return EDPC_OK;
+  return EDPC_OK;  // (Adam runs layer by layer within the backward pass)
 }
 
 // Step s of the delayed-update schedule (parity q = s % 2): the forward pass
@@ -1564,10 +1653,7 @@ int Model::step_delayed(const StepIO& io, cudaStream_t st) {
   const Parity& nxt = par[q ^ 1];
   if (io.update) {
     NoPdl scope;  // follows the join of bwd_st
-    if (precision != EDPC_FP32)
-      EDPC_CUDA(launch_adam_bf16(nxt.P, G, M, V, nxt.Pb, nparam, nxt.ctl, st, now.P));
-    else
-      EDPC_CUDA(launch_adam(nxt.P, G, M, V, nparam, nxt.ctl, st, now.P));
+    EDPC_CUDA(launch_adam(nxt.P, G, M, V, nxt.Pb, nparam, nxt.ctl, st, now.P));
   }
   if (io.advance) EDPC_CUDA(launch_step_advance(now.ctl, io.sp, d.K, io.ring_slots, d.b, st, nxt.ctl));
   select(q ^ 1);

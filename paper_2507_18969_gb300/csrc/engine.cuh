@@ -77,12 +77,11 @@ class Model {
   __nv_bfloat16 *dXpb = nullptr, *dXpbT = nullptr;
   float* dh0 = nullptr;                                    // gradient w.r.t. the embedding output
   TcPlan tcp;
-  cudaStream_t side = nullptr;                             // dW GEMMs and column sums
-  static constexpr int kForks = 4 * kMaxBlocks + 8;
+  cudaStream_t side = nullptr;                             // dW GEMMs
+  cudaStream_t side2 = nullptr;                            // column sums, and Adam layer by layer
+  static constexpr int kForks = 5 * kMaxBlocks + 16;
   cudaEvent_t fork[kForks] = {};
-  cudaEvent_t join_ev = nullptr;
   cudaEvent_t tr_ev = nullptr;                             // transposed weight copies ready
-  cudaEvent_t fdm_join_ev = nullptr;                       // side stream caught up before the FDM adjoint
   // FDM update off the critical path (BF16/FP8): dx' on the step's stream, the
   // Adam update of U, m, v on side_fdm from the pending copies; the next FDM
   // forward waits for adam_ev.
@@ -170,7 +169,6 @@ class Model {
   int forward(const StepIO& io, cudaStream_t st);
   int head(const StepIO& io, cudaStream_t st);
   int backward(const StepIO& io, cudaStream_t st);
-  int adam(cudaStream_t st);
   int step(const StepIO& io, cudaStream_t st);
   int step_delayed(const StepIO& io, cudaStream_t st);
   // Makes `st` wait for a pending FDM update (call before reading U, and before
@@ -217,9 +215,15 @@ class Model {
   size_t arena_bytes_ = 0;
   int nfork_ = 0;
   bool tuning_ = false;  // the tuner times the kernels that the tile codes name
+  Advance advance_of(const StepIO& io) const;
+  EmbAdam emb_adam(const StepIO& io) const;
+  int tile_lo[kMaxBlocks + 3] = {};  // first weight tile of each block, of the LTE, of the head; their end
+  int fork_to(cudaStream_t from, cudaStream_t to);
+  int adam_layer(const StepIO& io, int layer, cudaStream_t st);
+  int join_sides(cudaStream_t st);
   // FP32 path
   int block_fwd(int j, const float* Xin, float* Xout, cudaStream_t st);
-  int block_bwd(int j, float* dXnew, cudaStream_t st);
+  int block_bwd(const StepIO& io, int j, float* dXnew, cudaStream_t st);
   int side_f32(const float* dOut, int out, const float* X, int in, size_t w_off, ColsumJobs cj, cudaStream_t st);
   int forward_f32(const StepIO& io, cudaStream_t st);
   int backward_f32(const StepIO& io, cudaStream_t st);

@@ -938,6 +938,24 @@ cudaError_t launch_fdm_adam(const FdmSplitArgs& a, cudaStream_t st, bool persist
   }
 }
 
+__device__ __forceinline__ void advance_in_place(const Advance& a);
+
+// One value of dE, and Adam on its parameter (u.P == nullptr: the gradient only).
+__device__ __forceinline__ void emb_out(float* __restrict__ dE, const EmbAdam& u, size_t o, float g) {
+  dE[o] = g;
+  if (!u.P) return;
+  float p = u.P[o], m = u.M[o], v = u.V[o];
+  // adam1 with the contractions spelled out as the other parameters' Adam has
+  // them: beside the sums above the compiler contracted the other products
+  m = __fmaf_rn(kB1, m, __fmul_rn(1.0f - kB1, g));
+  v = __fmaf_rn(kB2, v, __fmul_rn(__fmul_rn(1.0f - kB2, g), g));
+  p = p - u.ctl->a_lr * (m / u.ctl->a_bc1) / (sqrtf(v / u.ctl->a_bc2) + kAdamEps);
+  u.P[o] = p;
+  u.M[o] = m;
+  u.V[o] = v;
+  if (u.Pb) u.Pb[o] = __float2bfloat16_rn(p);
+}
+
 // ============================================================================================
 // Embedding backward: scatter-add of dh0 into E's rows, owner computes.
 // CTA (c, q) owns byte value c and chunk q of kEmbChunkPos consecutive
@@ -1083,9 +1101,11 @@ template <int DT, class Scratch>
 __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __restrict__ ctx,
                                                               const float* __restrict__ dX, int P, int D,
                                                               float* __restrict__ dE, float* __restrict__ part,
-                                                              unsigned* __restrict__ cnt) {
+                                                              unsigned* __restrict__ cnt, Advance adv,
+                                                              EmbAdam upd) {
   pdl_wait();
   pdl_launch();
+  if (adv.ctl && blockIdx.x == 255 && blockIdx.y == 0 && threadIdx.x == 255) advance_in_place(adv);
   extern __shared__ __align__(16) unsigned char emb_smem[];
   Scratch* scratch = reinterpret_cast<Scratch*>(emb_smem);
   __shared__ float wsum[8][64];
@@ -1109,7 +1129,7 @@ __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __r
     for (int ww = 1; ww < 8; ++ww) sum += wsum[ww][t];
   }
   if (nq == 1) {
-    if (t < D) dE[(size_t)c * D + t] = sum;
+    if (t < D) emb_out(dE, upd, (size_t)c * D + t, sum);
     return;
   }
   if (t < D) {
@@ -1124,7 +1144,7 @@ __global__ void __launch_bounds__(256) embed_bwd_owner_kernel(const uint8_t* __r
     const float* src = part + (size_t)c * nq * D + t;
     float acc = 0.f;
     for (int k = 0; k < nq; ++k) acc += __ldcg(src + (size_t)k * D);
-    dE[(size_t)c * D + t] = acc;
+    emb_out(dE, upd, (size_t)c * D + t, acc);
     if (t == 0) cnt[c] = 0u;
   }
 }
@@ -1145,22 +1165,22 @@ static cudaError_t launch_emb_owner(dim3 grid, cudaStream_t st, A... args) {
 
 template <int DT>
 static cudaError_t launch_emb(dim3 grid, cudaStream_t st, const uint8_t* ctx, const float* dX, int P, int D, float* dE,
-                              float* part, unsigned* cnt) {
+                              float* part, unsigned* cnt, const Advance& adv, const EmbAdam& upd) {
   // 256 CTAs (one chunk) are resident at once with the deep ring; with several chunks more CTAs an SM count more
-  if (grid.y == 1) return launch_emb_owner<DT, EmbDeep>(grid, st, ctx, dX, P, D, dE, part, cnt);
-  return launch_emb_owner<DT, EmbWide>(grid, st, ctx, dX, P, D, dE, part, cnt);
+  if (grid.y == 1) return launch_emb_owner<DT, EmbDeep>(grid, st, ctx, dX, P, D, dE, part, cnt, adv, upd);
+  return launch_emb_owner<DT, EmbWide>(grid, st, ctx, dX, P, D, dE, part, cnt, adv, upd);
 }
 
 cudaError_t launch_embed_bwd(const uint8_t* ctx, const float* dX, int b, int K, int D, float* dE, float* part,
-                             unsigned* cnt, cudaStream_t st) {
+                             unsigned* cnt, const Advance& adv, const EmbAdam& upd, cudaStream_t st) {
   if (D > 64) return cudaErrorInvalidValue;
   const int nq = embed_bwd_chunks(b, K);
   if (nq > 1 && (!part || !cnt)) return cudaErrorInvalidValue;
   const dim3 grid(256, nq < 1 ? 1 : nq);
   switch (D) {  // the configurations' widths have their loops unrolled
-    case 8: return launch_emb<8>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
-    case 16: return launch_emb<16>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
-    default: return launch_emb<0>(grid, st, ctx, dX, b * K, D, dE, part, cnt);
+    case 8: return launch_emb<8>(grid, st, ctx, dX, b * K, D, dE, part, cnt, adv, upd);
+    case 16: return launch_emb<16>(grid, st, ctx, dX, b * K, D, dE, part, cnt, adv, upd);
+    default: return launch_emb<0>(grid, st, ctx, dX, b * K, D, dE, part, cnt, adv, upd);
   }
 }
 
@@ -1173,9 +1193,11 @@ template <int DT>
 __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __restrict__ ctx,
                                                                const float* __restrict__ dX, int K, int D,
                                                                float* __restrict__ dE,
-                                                               const GroupInfo* __restrict__ gi, size_t gs) {
+                                                               const GroupInfo* __restrict__ gi, size_t gs,
+                                                              Advance adv, EmbAdam upd) {
   pdl_wait();
   pdl_launch();
+  if (adv.ctl && blockIdx.x == 0 && blockIdx.y == 127 && threadIdx.x == 255) advance_in_place(adv);
   extern __shared__ __align__(16) unsigned char emb_smem[];
   EmbWide* scratch = reinterpret_cast<EmbWide*>(emb_smem);
   __shared__ float part[8][64];
@@ -1195,7 +1217,7 @@ __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __
   if ((w & 3) == 0) {
     const size_t o = (size_t)blockIdx.x * gs + (size_t)c * D;
     for (int d = lane; d < D; d += 32)
-      dE[o + d] = ((part[w][d] + part[w + 1][d]) + part[w + 2][d]) + part[w + 3][d];
+      emb_out(dE, upd, o + d, ((part[w][d] + part[w + 1][d]) + part[w + 2][d]) + part[w + 3][d]);
   }
 }
 
@@ -1212,14 +1234,15 @@ static cudaError_t launch_emb_groups(dim3 grid, cudaStream_t st, A... args) {
 }
 
 cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, int D, float* dE,
-                                    const GroupInfo* gi, int ngroups, size_t gs, cudaStream_t st) {
+                                    const GroupInfo* gi, int ngroups, size_t gs, const Advance& adv, const EmbAdam& upd,
+                                    cudaStream_t st) {
   if (D > 64 || ngroups < 1 || ngroups > 65535 || !gi || (reinterpret_cast<uintptr_t>(ctx) & 3))
     return cudaErrorInvalidValue;
   const dim3 grid(ngroups, 128);
   switch (D) {
-    case 8: return launch_emb_groups<8>(grid, st, ctx, dX, K, D, dE, gi, gs);
-    case 16: return launch_emb_groups<16>(grid, st, ctx, dX, K, D, dE, gi, gs);
-    default: return launch_emb_groups<0>(grid, st, ctx, dX, K, D, dE, gi, gs);
+    case 8: return launch_emb_groups<8>(grid, st, ctx, dX, K, D, dE, gi, gs, adv, upd);
+    case 16: return launch_emb_groups<16>(grid, st, ctx, dX, K, D, dE, gi, gs, adv, upd);
+    default: return launch_emb_groups<0>(grid, st, ctx, dX, K, D, dE, gi, gs, adv, upd);
   }
 }
 
@@ -1227,27 +1250,42 @@ cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, 
 // Adam on the shared parameters (Sec. 4.1: lr 1e-3; beta, eps as documented).
 // ============================================================================================
 // P is read from Pin and written to P (Pin == P: in place; the delayed-update
-// schedule writes the next parameters beside the current ones).
-__global__ void adam_kernel(float* P, const float* Pin, const float* __restrict__ G, float* __restrict__ M,
-                            float* __restrict__ V, size_t n, const StepCtl* __restrict__ ctl) {
+// schedule writes the next parameters beside the current ones). Pb: the BF16
+// copy, refreshed in the same pass. Four parameters a thread (tensor sizes are
+// multiples of 8): bound by loads in flight; with one parameter a thread the
+// 64 MiB mix's 2.0 M took 11.0 us, now 9.3. The whole set at once is the
+// delayed update's form; Algorithm 1's runs layer by layer (adam_layer_kernel).
+__global__ void __launch_bounds__(256) adam_kernel(float4* P, const float4* Pin, const float4* __restrict__ G,
+                                                   float4* __restrict__ M, float4* __restrict__ V,
+                                                   uint2* __restrict__ Pb, size_t n4, const StepCtl* __restrict__ ctl) {
   pdl_wait();
   pdl_launch();
-  const StepCtl c = *ctl;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    float p = Pin[e], m = M[e], v = V[e];
-    const float gr = G[e];
-    adam1(p, m, v, gr, c.lr, c.bc1, c.bc2);
+  const float lr = ctl->a_lr, bc1 = ctl->a_bc1, bc2 = ctl->a_bc2;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
+    float4 p = Pin[e], m = M[e], v = V[e];
+    const float4 g = G[e];
+    adam1(p.x, m.x, v.x, g.x, lr, bc1, bc2);
+    adam1(p.y, m.y, v.y, g.y, lr, bc1, bc2);
+    adam1(p.z, m.z, v.z, g.z, lr, bc1, bc2);
+    adam1(p.w, m.w, v.w, g.w, lr, bc1, bc2);
     P[e] = p;
     M[e] = m;
     V[e] = v;
+    if (Pb) {
+      __align__(8) __nv_bfloat162 h[2] = {__floats2bfloat162_rn(p.x, p.y), __floats2bfloat162_rn(p.z, p.w)};
+      Pb[e] = *reinterpret_cast<const uint2*>(h);
+    }
   }
 }
 
-cudaError_t launch_adam(float* P, const float* G, float* M, float* V, size_t n, const StepCtl* ctl,
+cudaError_t launch_adam(float* P, const float* G, float* M, float* V, __nv_bfloat16* Pb, size_t n, const StepCtl* ctl,
                         cudaStream_t st, const float* Pin) {
-  int grid = (int)((n + 255) / 256);
-  if (grid > 152 * 8) grid = 152 * 8;
-  return launch_k(adam_kernel, dim3(grid), dim3(256), 0, st, P, Pin ? Pin : P, G, M, V, n, ctl);
+  if (n & 3) return cudaErrorInvalidValue;
+  const size_t n4 = n / 4;
+  const int grid = (int)std::min<size_t>((n4 + 255) / 256, 152 * 8);
+  return launch_k(adam_kernel, dim3(grid), dim3(256), 0, st, reinterpret_cast<float4*>(P),
+                  reinterpret_cast<const float4*>(Pin ? Pin : P), reinterpret_cast<const float4*>(G),
+                  reinterpret_cast<float4*>(M), reinterpret_cast<float4*>(V), reinterpret_cast<uint2*>(Pb), n4, ctl);
 }
 
 // ============================================================================================
@@ -1276,6 +1314,21 @@ __device__ __forceinline__ StepCtl advance_ctl(StepCtl c, int dst_err, Split sp,
   c.bc2 = 1.0f - powf(kB2, (float)c.t);
   c.slot = (int)((i - K) % ring_slots);
   return c;
+}
+
+// In place, by one thread of a launch that no reader of the record overlaps but
+// Adam, which reads its own copy of the scalars (a_*), and kernels that set
+// error bits (which are left alone).
+__device__ __forceinline__ void advance_in_place(const Advance& a) {
+  const StepCtl c = advance_ctl(*a.ctl, 0, a.sp, a.K, a.ring_slots, a.b);
+  a.ctl->i = c.i;
+  a.ctl->t = c.t;
+  a.ctl->bact = c.bact;
+  a.ctl->slot = c.slot;
+  a.ctl->inv_bact = c.inv_bact;
+  a.ctl->bc1 = c.bc1;
+  a.ctl->bc2 = c.bc2;
+  a.ctl->cpi = c.cpi;
 }
 
 __global__ void step_advance_kernel(const StepCtl* src, StepCtl* dst, Split sp, int K, int ring_slots, int b) {
@@ -1682,6 +1735,11 @@ __global__ void __launch_bounds__(32 * kRowsHead) head_kernel(HeadArgs a) {
   }
   pdl_wait();
   pdl_launch();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // Adam's scalars of this step
+    a.ctl->a_lr = c.lr;
+    a.ctl->a_bc1 = c.bc1;
+    a.ctl->a_bc2 = c.bc2;
+  }
   float dzv[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) dzv[q] = 0.f;
@@ -2343,32 +2401,84 @@ cudaError_t launch_colsum_groups(const ColsumJobs& jobs, const GroupInfo* gi, in
 }
 
 // ============================================================================================
-// Adam with the BF16 weight copy refreshed in the same pass; transposed copies
-// of every weight matrix in one launch (32 x 32 tiles through shared memory).
+// Adam of one layer's parameters with both BF16 copies of its weights: CTA = one
+// 32 x 32 tile of a weight matrix (four parameters a thread; the updated tile
+// goes through shared memory into the transposed copy) or 1024 entries of the
+// layer's bias and LayerNorm vectors; grid y = group (grouped mode).
+// A layer's launch (5 us for the 0.4 M parameters of a block of the 64 MiB mix)
+// follows its gradients on a side stream, so most of the update hides under the
+// rest of the adjoint, and the transposed copies need no pass of their own at
+// the next step's start (8.5 us there, 56 us for 12 independent models).
 // ============================================================================================
-__global__ void adam_bf16_kernel(float* P, const float* Pin, const float* __restrict__ G, float* __restrict__ M,
-                                 float* __restrict__ V, __nv_bfloat16* __restrict__ Pb, size_t n,
-                                 const StepCtl* __restrict__ ctl) {
+__global__ void __launch_bounds__(256) adam_layer_kernel(AdamLayer a) {
   pdl_wait();
   pdl_launch();
-  const StepCtl c = *ctl;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    float p = Pin[e], m = M[e], v = V[e];
-    const float gr = G[e];
-    adam1(p, m, v, gr, c.lr, c.bc1, c.bc2);
-    P[e] = p;
-    M[e] = m;
-    V[e] = v;
-    Pb[e] = __float2bfloat16_rn(p);
+  __shared__ __nv_bfloat16 t[32][34];
+  const float lr = a.ctl->a_lr, bc1 = a.ctl->a_bc1, bc2 = a.ctl->a_bc2;
+  const size_t go = (size_t)blockIdx.y * a.gs;  // the group's parameters
+  auto update = [&](size_t e) -> float4 {        // four parameters at e
+    e += go;
+    float4 p = *reinterpret_cast<float4*>(a.P + e), m = *reinterpret_cast<float4*>(a.M + e),
+           v = *reinterpret_cast<float4*>(a.V + e);
+    const float4 g = *reinterpret_cast<const float4*>(a.G + e);
+    adam1(p.x, m.x, v.x, g.x, lr, bc1, bc2);
+    adam1(p.y, m.y, v.y, g.y, lr, bc1, bc2);
+    adam1(p.z, m.z, v.z, g.z, lr, bc1, bc2);
+    adam1(p.w, m.w, v.w, g.w, lr, bc1, bc2);
+    *reinterpret_cast<float4*>(a.P + e) = p;
+    *reinterpret_cast<float4*>(a.M + e) = m;
+    *reinterpret_cast<float4*>(a.V + e) = v;
+    if (a.Pb) {
+      __align__(8) __nv_bfloat162 h[2] = {__floats2bfloat162_rn(p.x, p.y), __floats2bfloat162_rn(p.z, p.w)};
+      *reinterpret_cast<uint2*>(a.Pb + e) = *reinterpret_cast<const uint2*>(h);
+    }
+    return p;
+  };
+  if ((int)blockIdx.x < a.ntiles) {  // CTA-uniform
+    const TransposeTile tl = a.tiles[blockIdx.x];
+    const int y = threadIdx.x >> 3, x = (threadIdx.x & 7) * 4;  // rows and columns are multiples of 8
+    if (tl.r0 + y < tl.rows && tl.c0 + x < tl.cols) {
+      const float4 p = update(tl.off + (size_t)(tl.r0 + y) * tl.cols + tl.c0 + x);
+      t[y][x] = __float2bfloat16_rn(p.x);
+      t[y][x + 1] = __float2bfloat16_rn(p.y);
+      t[y][x + 2] = __float2bfloat16_rn(p.z);
+      t[y][x + 3] = __float2bfloat16_rn(p.w);
+    }
+    __syncthreads();
+    // y: column, x: four rows
+    if (tl.c0 + y < tl.cols && tl.r0 + x < tl.rows) {
+      __align__(8) __nv_bfloat16 h[4] = {t[x][y], t[x + 1][y], t[x + 2][y], t[x + 3][y]};
+      *reinterpret_cast<uint2*>(a.PbT + go + tl.off + (size_t)(tl.c0 + y) * tl.rows + tl.r0 + x) =
+          *reinterpret_cast<const uint2*>(h);
+    }
+    return;
+  }
+  // entry e4 of the layer's vectors, laid end to end
+  size_t e = ((size_t)(blockIdx.x - a.ntiles) * 256 + threadIdx.x) * 4;
+  for (int q = 0; q < a.nvec; ++q) {
+    if (e < a.vec[q].n) {
+      update(a.vec[q].off + e);
+      return;
+    }
+    e -= a.vec[q].n;
   }
 }
-cudaError_t launch_adam_bf16(float* P, const float* G, float* M, float* V, __nv_bfloat16* Pb, size_t n,
-                             const StepCtl* ctl, cudaStream_t st, const float* Pin) {
-  int grid = (int)((n + 255) / 256);
-  if (grid > 152 * 8) grid = 152 * 8;
-  return launch_k(adam_bf16_kernel, dim3(grid), dim3(256), 0, st, P, Pin ? Pin : P, G, M, V, Pb, n, ctl);
+
+cudaError_t launch_adam_layer(const AdamLayer& a, cudaStream_t st) {
+  size_t nv = 0;
+  for (int q = 0; q < a.nvec; ++q) {
+    if ((a.vec[q].n | a.vec[q].off) & 3) return cudaErrorInvalidValue;
+    nv += a.vec[q].n;
+  }
+  const size_t grid = a.ntiles + (nv + 1023) / 1024;
+  if (grid == 0) return cudaSuccess;
+  if (grid > 0x7fffffffu) return cudaErrorInvalidValue;
+  return launch_k(adam_layer_kernel, dim3((unsigned)grid, a.groups), dim3(256), 0, st, a);
 }
 
+// ============================================================================================
+// Transposed copies of every weight matrix in one launch (32 x 32 tiles through shared memory).
+// ============================================================================================
 __global__ void transpose_tiles_kernel(const __nv_bfloat16* __restrict__ Pb, __nv_bfloat16* __restrict__ PbT,
                                        const TransposeTile* __restrict__ tiles, int ntiles) {
   pdl_wait();

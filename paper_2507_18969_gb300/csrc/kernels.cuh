@@ -43,7 +43,7 @@ cudaError_t launch_fdm_fwd(const float* Xp, const float* U, float* Y, int b, int
 struct HeadArgs {
   const float* z;            // b x 256 logits
   int b;
-  const StepCtl* ctl;
+  StepCtl* ctl;              // read; also gets Adam's scalars of the step (a_*)
   Split sp;
   int mode;                  // 0 encode, 1 decode, 2 model API (targets/active given)
   uint8_t* data;             // stream bytes (read at encode, written at decode)
@@ -144,21 +144,37 @@ cudaError_t launch_fdm_adam(const FdmSplitArgs& a, cudaStream_t st, bool persist
 // more than one chunk, part (256 * chunks * D floats) and cnt (256 counters,
 // zero between launches) hold the chunk partials; launches sharing them must
 // not overlap.
+// adv.ctl != nullptr: the launch also advances the step control in place (its
+// only later reader in the step is Adam, which reads a_*).
+struct Advance {
+  StepCtl* ctl = nullptr;
+  Split sp{};
+  int K = 0, ring_slots = 1, b = 0;
+};
+// upd.P != nullptr: Adam on the table (P, M, V, and its BF16 copy Pb) in the
+// same launch, with the scalars a_* of ctl; grouped mode: offset by g * gs.
+struct EmbAdam {
+  float *P = nullptr, *M = nullptr, *V = nullptr;
+  __nv_bfloat16* Pb = nullptr;
+  const StepCtl* ctl = nullptr;
+};
 constexpr int kEmbChunkPos = 16384;
 int embed_bwd_chunks(int b, int K);
 cudaError_t launch_embed_bwd(const uint8_t* ctx, const float* dX, int b, int K, int D, float* dE, float* part,
-                             unsigned* cnt, cudaStream_t st);
+                             unsigned* cnt, const Advance& adv, const EmbAdam& upd, cudaStream_t st);
 // Grouped mode: dE of group g (at dE + g * gs) sums the positions of its
 // stream rows [gi[g].r0, gi[g].r0 + gi[g].s) only, in a fixed order that
 // depends on the group alone (four quarters of the positions, each summed in
 // increasing order, then added in order); CTAs per group and pair of byte
 // values (ctx 4-byte aligned).
 cudaError_t launch_embed_bwd_groups(const uint8_t* ctx, const float* dX, int K, int D, float* dE,
-                                    const GroupInfo* gi, int ngroups, size_t gs, cudaStream_t st);
+                                    const GroupInfo* gi, int ngroups, size_t gs, const Advance& adv, const EmbAdam& upd,
+                                    cudaStream_t st);
 
-// Adam over the flat shared parameters; bf16 != nullptr also refreshes the BF16 copy.
-// Pin: the parameters read (nullptr: P itself, an in-place update).
-cudaError_t launch_adam(float* P, const float* G, float* M, float* V, size_t n, const StepCtl* ctl,
+// Adam over n (a multiple of 4) shared parameters at 16-byte aligned pointers;
+// Pb != nullptr also refreshes their BF16 copy. Pin: the parameters read
+// (nullptr: P itself, an in-place update). Reads the scalars a_* of ctl.
+cudaError_t launch_adam(float* P, const float* G, float* M, float* V, __nv_bfloat16* Pb, size_t n, const StepCtl* ctl,
                         cudaStream_t st, const float* Pin = nullptr);
 // i += 1 and the derived per-step scalars.
 // dst: where the next step's control goes (nullptr: ctl itself).
@@ -260,9 +276,6 @@ cudaError_t launch_colsum_multi(const ColsumJobs& jobs, cudaStream_t st);
 // rows hold zero gradients; chunk fields of jobs unused).
 cudaError_t launch_colsum_groups(const ColsumJobs& jobs, const GroupInfo* gi, int ngroups, size_t gs,
                                  cudaStream_t st);
-// Adam that also writes the BF16 copy Pb of every updated parameter (same flat layout).
-cudaError_t launch_adam_bf16(float* P, const float* G, float* M, float* V, __nv_bfloat16* Pb, size_t n,
-                             const StepCtl* ctl, cudaStream_t st, const float* Pin = nullptr);
 // Transposed BF16 copies of several matrices in one launch: PbT[off + c*rows + r] = Pb[off + r*cols + c].
 struct TransposeTile {
   unsigned long long off;
@@ -270,6 +283,24 @@ struct TransposeTile {
 };
 cudaError_t launch_transpose_tiles(const __nv_bfloat16* Pb, __nv_bfloat16* PbT, const TransposeTile* tiles,
                                    int ntiles, cudaStream_t st);
+// Adam of one layer: the weight matrices cut into `tiles` (device array; both
+// BF16 copies written) and the flat ranges vec (Pb written when non-null),
+// offsets into P, G, M, V, Pb and PbT; group g's parameters at + g * gs.
+struct AdamLayer {
+  float *P = nullptr, *M = nullptr, *V = nullptr;
+  const float* G = nullptr;
+  __nv_bfloat16 *Pb = nullptr, *PbT = nullptr;
+  const TransposeTile* tiles = nullptr;
+  int ntiles = 0;
+  struct Range {
+    size_t off, n;  // multiples of 4
+  } vec[8] = {};
+  int nvec = 0;
+  unsigned groups = 1;
+  size_t gs = 0;
+  const StepCtl* ctl = nullptr;
+};
+cudaError_t launch_adam_layer(const AdamLayer& a, cudaStream_t st);
 
 // ---- BF16 operands ------------------------------------------------------------------------------
 // Y[r][c] = bf16(X[r][c]) (ld ldy) and/or YT[c][r] = bf16(X[r][c]) (ld ldt).

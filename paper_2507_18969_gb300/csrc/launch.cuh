@@ -28,6 +28,13 @@ struct NoPdl {
   ~NoPdl() { g_pdl_enabled = saved; }
 };
 
+// Keeps the attribute as it is when `on`, else turns it off for the scope.
+struct PdlScope {
+  bool saved;
+  explicit PdlScope(bool on) : saved(g_pdl_enabled) { g_pdl_enabled = saved && on; }
+  ~PdlScope() { g_pdl_enabled = saved; }
+};
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_k(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                             Args&&... args) {
