@@ -1,10 +1,10 @@
 // BF16 / FP8 GEMM on the 5th-generation tensor cores (sm_103a).
 //
 // One CTA computes a 128 x BN tile of C = A B^T:
-//   warp 8 (one lane)  issues TMA loads of 128-byte-wide A (128 rows) and B
+//   warp 8 (a lane)    issues TMA loads of 128-byte-wide A (128 rows) and B
 //                      (BN rows) tiles (64 BF16 or 128 FP8 elements of K,
 //                      128-byte swizzle) into a STAGES-deep ring;
-//   warp 9 (one lane)  issues tcgen05.mma (M=128, N=BN; kind::f16 with K=16
+//   warp 9 (a lane)    issues tcgen05.mma (M=128, N=BN; kind::f16 with K=16
 //                      for BF16, kind::f8f6f4 with K=32 for FP8 e4m3; FP32
 //                      accumulation) into a TMEM accumulator and commits each
 //                      stage back to its "empty" barrier, and allocates / frees
@@ -137,10 +137,13 @@ __global__ void __launch_bounds__(kTcThreads, MODE == TC_PLAIN || BN > 64 ? 2 : 
     }
   };
   const int npre = e.b_early ? (nk < STAGES ? nk : STAGES) : 0;
-  if (warp == 8 && lane == 0) {
+  if (warp == 8) {
     for (int kb = 0; kb < npre; ++kb) {
-      mbar_expect_tx(&full[kb], A_BYTES + B_BYTES);
-      load_b(kb, kb);
+      if (elect_one()) {
+        mbar_expect_tx(&full[kb], A_BYTES + B_BYTES);
+        load_b(kb, kb);
+      }
+      __syncwarp();
     }
   }
   // The epilogue's view of the problem; grouped mode: the tile's row bound, its
@@ -164,38 +167,46 @@ __global__ void __launch_bounds__(kTcThreads, MODE == TC_PLAIN || BN > 64 ? 2 : 
   pdl_wait();
   pdl_launch();
 
-  if (warp == 8 && lane == 0) {
+  if (warp == 8) {
     // TMA producer
+    int s = 0;
+    uint32_t ph = 1;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-      if (kb >= STAGES && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
-      if (kb >= npre) {
-        mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-        load_b(kb, s);
+      if (kb >= STAGES && !warp_wait(&empty[s], ph, abort_flag)) break;
+      if (elect_one()) {
+        if (kb >= npre) {
+          mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
+          load_b(kb, s);
+        }
+        tma_load_2d(sA + s * A_BYTES, &ta, kel0 + (kb_lo + kb) * BK, m0, &full[s]);
       }
-      tma_load_2d(sA + s * A_BYTES, &ta, kel0 + (kb_lo + kb) * BK, m0, &full[s]);
+      __syncwarp();
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
-  } else if (warp == 9 && lane == 0) {
+  } else if (warp == 9) {
     // MMA issuer
     constexpr uint32_t idesc = F8 ? idesc_e4m3(BN) : idesc_bf16(BN);
+    const uint32_t ad = desc_lo(sA), bd = desc_lo(sB);
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (uint32_t)(kb / STAGES) & 1u;
-      if (!mbar_wait(&full[s], ph, abort_flag)) break;
+      if (!warp_wait(&full[s], ph, abort_flag)) break;
       tc_fence_after();
-#pragma unroll
-      for (int k = 0; k < BKB / 32; ++k) {  // one MMA per 32 bytes of K
-        const uint64_t ad = sdesc(sA + s * A_BYTES + k * 32);
-        const uint64_t bd = sdesc(sB + s * B_BYTES + k * 32);
-        if (F8)
-          mma_e4m3(tmem, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-        else
-          mma_bf16(tmem, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+      if (elect_one()) {
+        mma_stage<F8>(tmem, ad + s * (A_BYTES >> 4), bd + s * (B_BYTES >> 4), idesc, kb == 0);
+        if (kb + STAGES < nk) mma_commit(&empty[s]);  // (else nothing waits for the stage)
       }
-      mma_commit(&empty[s]);
+      __syncwarp();
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
-    mma_commit(done);
+    __syncwarp();
+    if (elect_one()) mma_commit(done);
   }
   __syncwarp();
 

@@ -88,6 +88,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// The same by a whole warp, with one answer for all its lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
@@ -108,18 +113,23 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, in
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// K-major operand tile with 128-byte swizzle: rows of 128 bytes, 8-row groups
-// 1024 bytes apart (stride byte offset), descriptor version 1, layout 2.
-__device__ __forceinline__ uint64_t sdesc(const void* p) {
-  uint64_t a = smem_u32(p);
-  uint64_t d = 0;
-  d |= (a & 0x3FFFFull) >> 4;
-  d |= (uint64_t)(16 >> 4) << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
+// One lane of a converged warp. The issuing warps run their loops as whole warps
+// and elect a lane around each instruction: loop counters, addresses and
+// descriptors then stay in uniform registers, where TMA and MMA instructions
+// take them from. With the loops inside `if (lane == 0)` every one of them was
+// moved over from vector registers: a 64-wide K block of a 128 x 32 tile took 685
+// cycles, now 429.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+  return p != 0;
 }
+
+// Shared-memory descriptor of a K-major operand tile with 128-byte swizzle: rows
+// of 128 bytes, 8-row groups 1024 bytes apart (stride byte offset), descriptor
+// version 1, layout 2. Its upper half is the same for every tile.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(const void* p) { return ((smem_u32(p) & 0x3FFFFu) >> 4) | (1u << 16); }
 
 // Instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = bn.
 __host__ __device__ constexpr uint32_t idesc_bf16(int bn) {
@@ -130,18 +140,32 @@ __host__ __device__ constexpr uint32_t idesc_e4m3(int bn) {
   return (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
+// ad, bd: lower halves of the operands' descriptors.
+__device__ __forceinline__ void mma_bf16(uint32_t dtm, uint32_t ad, uint32_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(dtm),
+      "r"(ad), "r"(bd), "r"(idesc), "r"(acc), "n"(kDescHi));
 }
 
-__device__ __forceinline__ void mma_e4m3(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_e4m3(uint32_t dtm, uint32_t ad, uint32_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+      " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a, b, %3, p;\n}\n" ::"r"(dtm),
+      "r"(ad), "r"(bd), "r"(idesc), "r"(acc), "n"(kDescHi));
+}
+
+// The MMAs of one stage (128 bytes of K, 32 a piece), by one elected lane.
+template <bool F8>
+__device__ __forceinline__ void mma_stage(uint32_t dtm, uint32_t ad, uint32_t bd, uint32_t idesc, bool first) {
+#pragma unroll
+  for (int k = 0; k < BKB / 32; ++k) {
+    const uint32_t acc = (k > 0 || !first) ? 1u : 0u;
+    if (F8)
+      mma_e4m3(dtm, ad + 2 * k, bd + 2 * k, idesc, acc);
+    else
+      mma_bf16(dtm, ad + 2 * k, bd + 2 * k, idesc, acc);
+  }
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {

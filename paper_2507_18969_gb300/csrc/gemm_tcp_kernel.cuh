@@ -120,19 +120,18 @@ __global__ void __launch_bounds__(192, 1)
   pdl_launch();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // TMA producer
-      uint32_t it = 0;
-      bool go = true;
-      for (int u = cid; u < nunits && go; u += ncl) {
-        const Tile q = decode(u);
-        for (int kb = 0; kb < q.nk; ++kb, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (it / STAGES) & 1u;
-          if (it >= (uint32_t)STAGES && !mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
-            go = false;
-            break;
-          }
+    // TMA producer
+    int s = 0;
+    uint32_t ph = 1, it = 0;
+    bool go = true;
+    for (int u = cid; u < nunits && go; u += ncl) {
+      const Tile q = decode(u);
+      for (int kb = 0; kb < q.nk; ++kb, ++it) {
+        if (it >= (uint32_t)STAGES && !warp_wait(&empty[s], ph, abort_flag)) {
+          go = false;
+          break;
+        }
+        if (elect_one()) {
           mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
           const int kc = (q.lo + kb) * BK;
 #pragma unroll
@@ -142,43 +141,46 @@ __global__ void __launch_bounds__(192, 1)
           }
           tma_load_2d(sA + s * A_BYTES, &ta, kc, q.m0, &full[s]);
         }
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      constexpr uint32_t idesc = F8 ? idesc_e4m3(BN) : idesc_bf16(BN);
-      uint32_t it = 0;
-      int tcount = 0;
-      bool go = true;
-      for (int u = cid; u < nunits && go; u += ncl, ++tcount) {
-        const Tile q = decode(u);
-        const int a = tcount & 1;
-        // accumulator a was last used by tile tcount - 2: wait until it is drained
-        if (tcount >= 2 && !mbar_wait(&tempty[a], (uint32_t)((tcount >> 1) - 1) & 1u, abort_flag)) break;
+    // MMA issuer
+    constexpr uint32_t idesc = F8 ? idesc_e4m3(BN) : idesc_bf16(BN);
+    const uint32_t ad = desc_lo(sA), bd = desc_lo(sB);
+    int s = 0;
+    uint32_t ph = 0;
+    int tcount = 0;
+    bool go = true;
+    for (int u = cid; u < nunits && go; u += ncl, ++tcount) {
+      const Tile q = decode(u);
+      const int a = tcount & 1;
+      // accumulator a was last used by tile tcount - 2: wait until it is drained
+      if (tcount >= 2 && !warp_wait(&tempty[a], (uint32_t)((tcount >> 1) - 1) & 1u, abort_flag)) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + (uint32_t)a * ACC;
+      for (int kb = 0; kb < q.nk; ++kb) {
+        if (!warp_wait(&full[s], ph, abort_flag)) {
+          go = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t dt = tmem + (uint32_t)a * ACC;
-        for (int kb = 0; kb < q.nk; ++kb, ++it) {
-          const int s = (int)(it % STAGES);
-          const uint32_t ph = (it / STAGES) & 1u;
-          if (!mbar_wait(&full[s], ph, abort_flag)) {
-            go = false;
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int k = 0; k < BKB / 32; ++k) {  // one MMA per 32 bytes of K
-            const uint64_t ad = sdesc(sA + s * A_BYTES + k * 32);
-            const uint64_t bd = sdesc(sB + s * B_BYTES + k * 32);
-            if (F8)
-              mma_e4m3(dt, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-            else
-              mma_bf16(dt, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          }
+        if (elect_one()) {
+          mma_stage<F8>(dt, ad + s * (A_BYTES >> 4), bd + s * (B_BYTES >> 4), idesc, kb == 0);
           mma_commit(&empty[s]);
         }
-        if (go) mma_commit(&tfull[a]);
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
+      if (go && elect_one()) mma_commit(&tfull[a]);
+      __syncwarp();
     }
   } else {
     // epilogue warps 2-5; tcgen05.ld lets warp w reach TMEM lanes 32(w%4)..+31

@@ -14,15 +14,19 @@
 // is one value a lane, and no output passes through shared memory.
 //
 // At 512 streams, F = 512, H = 256, in the step (one-tile kernel before): branch
-// GEMM 5.7 -> 5.2 us, its adjoint 6.1 -> 4.8, out GEMM 3.7 -> 3.2, head 5.4 -> 4.3.
+// GEMM 5.7 -> 5.2 us, its adjoint 6.1 -> 4.8, out GEMM 3.7 -> 3.2, head 5.4 -> 4.3;
+// and, back to back, branch GEMM 5.8 -> 4.8, adjoint 6.6 -> 5.7, a plain K = 512
+// 4.9 -> 4.0 once the issuing warps ran as whole warps (elect_one). What is left
+// is the chain: 0.35 us until the first stage lands, 0.22 us a K block of 64 for
+// its four MMAs, 0.4 to 1.3 us of epilogue, and the hand-over between launches.
 //
 // Per element the products, their order over K and the epilogue's operations
 // are those of gemm_tc_kernel, and so are the results, bit for bit.
 //
-//   warp 8 (one lane)  TMA loads into an 8-stage ring: 128 rows of W (in the
+//   warp 8 (a lane)    TMA loads into an 8-stage ring: 128 rows of W (in the
 //                      branch GEMM 128 / k rows of each branch's section, 32
 //                      for k = 3) and NS rows of X, 64 BF16 of K a stage;
-//   warp 9 (one lane)  tcgen05.mma (M = 128, N = NS), TMEM allocation;
+//   warp 9 (a lane)    tcgen05.mma (M = 128, N = NS), TMEM allocation;
 //   warps 0-7          epilogue: warp w reads lanes 32 (w & 3) .. of the columns
 //                      of half w >> 2; loads that do not depend on the
 //                      accumulator, and GELU's derivative, come before.
@@ -110,8 +114,12 @@ __global__ void __launch_bounds__(kThreadsS, 1)
     for (int i = 0; i < SECTIONS; ++i)
       tma_load_2d(sW + s * W_BYTES + i * (SR * BKB), &tw, kb * 64, (MODE == TC_BRANCH ? i * e.H : 0) + n0, &full[s]);
   };
-  if (warp == 8 && lane == 0)
-    for (int kb = 0; kb < nk && kb < nst; ++kb) load_w(kb, kb);
+  if (warp == 8) {
+    for (int kb = 0; kb < nk && kb < nst; ++kb) {
+      if (elect_one()) load_w(kb, kb);
+      __syncwarp();
+    }
+  }
 
   // The epilogue's inputs besides the accumulator (written two or more
   // launches ago): the lane's bias, the residual or the saved branch outputs.
@@ -141,30 +149,41 @@ __global__ void __launch_bounds__(kThreadsS, 1)
   pdl_wait();
   pdl_launch();
 
-  if (warp == 8 && lane == 0) {
+  if (warp == 8) {
+    int s = 0;
+    uint32_t ph = 1;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % nst;
-      const uint32_t ph = (uint32_t)(kb / nst) & 1u;
-      if (kb >= nst) {
-        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
-        load_w(kb, s);
+      if (kb >= nst && !warp_wait(&empty[s], ph, abort_flag)) break;
+      if (elect_one()) {
+        if (kb >= nst) load_w(kb, s);
+        tma_load_2d(sX + s * X_BYTES, &tx, kb * 64, m0, &full[s]);
       }
-      tma_load_2d(sX + s * X_BYTES, &tx, kb * 64, m0, &full[s]);
+      __syncwarp();
+      if (++s == nst) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
-  } else if (warp == 9 && lane == 0) {
+  } else if (warp == 9) {
     constexpr uint32_t idesc = idesc_bf16(NS);
+    const uint32_t ad = desc_lo(sW), bd = desc_lo(sX);
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % nst;
-      const uint32_t ph = (uint32_t)(kb / nst) & 1u;
-      if (!mbar_wait(&full[s], ph, abort_flag)) break;
+      if (!warp_wait(&full[s], ph, abort_flag)) break;
       tc_fence_after();
-#pragma unroll
-      for (int k = 0; k < BKB / 32; ++k)
-        mma_bf16(tmem, sdesc(sW + s * W_BYTES + k * 32), sdesc(sX + s * X_BYTES + k * 32), idesc,
-                 (kb > 0 || k > 0) ? 1u : 0u);
-      mma_commit(&empty[s]);
+      if (elect_one()) {
+        mma_stage<false>(tmem, ad + s * (W_BYTES >> 4), bd + s * (X_BYTES >> 4), idesc, kb == 0);
+        if (kb + nst < nk) mma_commit(&empty[s]);  // (else nothing waits for the stage)
+      }
+      __syncwarp();
+      if (++s == nst) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
-    mma_commit(done);
+    __syncwarp();
+    if (elect_one()) mma_commit(done);
   }
   __syncwarp();
 
