@@ -322,7 +322,6 @@ int Model::init(const edpc_cfg& cfg, int streams, const std::vector<GroupInfo>* 
       }
     }
     if (!bf16) {
-      dG = a.take<float>(bH);
       for (int j = 0; j < d.n; ++j) {
         bb[j].dOut = a.take<float>(bF);
         bb[j].dA = a.take<float>(bkH);
@@ -565,19 +564,21 @@ int Model::refresh_bf16_weights(cudaStream_t st) {
 int Model::linear_fwd(const float* X, int rows, int in, size_t w_off, size_t b_off, int out, const float* resid,
                       float* Yo, cudaStream_t st) {
   const int epi = resid ? EPI_BIAS_RESID : EPI_BIAS;
-  GemmF32 g{rows, out, in, X, in, true, P + w_off, in, true, Yo, out, epi, P + b_off, resid, out, true};
+  GemmF32 g{rows, out, in, X, in, true, P + w_off, in, true, Yo, out, epi, P + b_off, resid, out};
+  g.b_early = true;
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }
 
 int Model::linear_dx(const float* dOut, int rows, int out, size_t w_off, int in, float* dX, cudaStream_t st) {
-  GemmF32 g{rows, in, out, dOut, out, true, P + w_off, in, false, dX, in, EPI_STORE, nullptr, nullptr, 0, true};
+  GemmF32 g{rows, in, out, dOut, out, true, P + w_off, in, false, dX, in, EPI_STORE, nullptr, nullptr, 0};
+  g.b_early = true;
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }
 
 int Model::linear_dw(const float* dOut, int rows, int out, const float* X, int in, size_t w_off, cudaStream_t st) {
-  GemmF32 g{out, in, rows, dOut, out, false, X, in, false, G + w_off, in, EPI_STORE, nullptr, nullptr, 0, false};
+  GemmF32 g{out, in, rows, dOut, out, false, X, in, false, G + w_off, in, EPI_STORE, nullptr, nullptr, 0};
   EDPC_CUDA(launch_gemm_f32(g, st));
   return EDPC_OK;
 }
@@ -587,8 +588,13 @@ int Model::block_fwd(int j, const float* Xin, float* Xout, cudaStream_t st) {
   BlockAct& a = ba[j];
   const int kH = d.k * d.H;
   EDPC_CUDA(launch_ln_fwd(Xin, P + o.ln_g, P + o.ln_b, a.xhat, a.rstd, a.X0, d.b, d.F, st));  // Eq. 9
-  EDPC_TRY(linear_fwd(a.X0, d.b, d.F, o.W, o.c, kH, nullptr, a.A, st));                       // Eq. 10
-  EDPC_CUDA(launch_branch_gelu(a.A, d.b, d.H, d.k, a.G, st));                                 // Eqs. 11-12
+  {  // Eqs. 10-12
+    GemmF32 g{d.b, d.H, d.F, a.X0, d.F, true, P + o.W, d.F, true, a.A, kH, EPI_BRANCH, P + o.c, nullptr, 0};
+    g.k = d.k;
+    g.G2 = a.G;
+    g.b_early = true;
+    EDPC_CUDA(launch_gemm_f32(g, st));
+  }
   EDPC_TRY(linear_fwd(a.G, d.b, d.H, o.Wo, o.co, d.F, Xin, Xout, st));                        // Eq. 13
   return EDPC_OK;
 }
@@ -649,9 +655,12 @@ int Model::block_bwd(const StepIO& io, int j, float* dXnew, cudaStream_t st) {
   const int kH = d.k * d.H;
   // Eq. 13: out = G Wo^T + co + X
   EDPC_TRY(side_f32(q.dOut, d.F, a.G, d.H, o.Wo, ColsumJobs{}, st));
-  EDPC_TRY(linear_dx(q.dOut, d.b, d.F, o.Wo, d.H, dG, st));
-  // Eqs. 11-12: G = GELU(prod X_i)
-  EDPC_CUDA(launch_branch_gelu_bwd(dG, a.A, d.b, d.H, d.k, q.dA, st));
+  {  // its input's gradient, and the adjoint of Eqs. 11-12 on it: G = GELU(prod X_i)
+    GemmF32 g{d.b, d.H, d.F, q.dOut, d.F, true, P + o.Wo, d.H, false, q.dA, kH, EPI_BRANCH_BWD, nullptr, a.A, kH};
+    g.k = d.k;
+    g.b_early = true;
+    EDPC_CUDA(launch_gemm_f32(g, st));
+  }
   // Eq. 10: X_i = X0 W_i^T + c_i
   EDPC_TRY(side_f32(q.dA, kH, a.X0, d.F, o.W, ColsumJobs{}, st));
   EDPC_TRY(linear_dx(q.dA, d.b, kH, o.W, d.F, q.dX0, st));

@@ -49,7 +49,6 @@ class Model {
   float* S[kMaxBlocks + 2] = {};          // residual-stream stages, b x F
   BlockAct ba[kMaxBlocks] = {};
   float *Xp = nullptr, *Y = nullptr, *z = nullptr, *p = nullptr, *dz = nullptr;
-  float* dG = nullptr;                    // FP32 path: gradient w.r.t. a block's GELU output
   float *dY = nullptr, *dXp = nullptr;
   float* emb_part = nullptr;              // embedding-adjoint chunk partials (many positions)
   unsigned* emb_cnt = nullptr;            // their arrival counters, one per byte value

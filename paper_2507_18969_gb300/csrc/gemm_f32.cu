@@ -22,6 +22,12 @@ namespace {
 
 constexpr int BKT = 32;
 
+// Exact erf GELU and its derivative (Eqs. 11-12 and their adjoint).
+__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
+__device__ __forceinline__ float gelu_grad_f(float x) {
+  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
+}
+
 __device__ __forceinline__ void cp16(float* dst, const float* src, int bytes) {  // bytes < 16: zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
                    static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
@@ -98,20 +104,25 @@ struct Operand {
   }
 };
 
-template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK>
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int KB>
 struct Tile {
   using A = Operand<AK, BM, TM>;
   using B = Operand<BK, BN, TN>;
   static constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
   static constexpr int WX = TX < 8 ? TX : 8, WY = 32 / WX;  // threads of a warp along n and m
   static_assert(NT % 32 == 0 && TX % WX == 0 && TY % WY == 0, "whole warps");
-  static constexpr int STAGE = A::FLOATS + B::FLOATS;
+  static constexpr int STAGE = A::FLOATS + KB * B::FLOATS;  // KB: sections of B (branches)
   static constexpr size_t kSmem = (size_t)STAGES * STAGE * sizeof(float);
 };
 
-template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI>
-__global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm_f32_kernel(const GemmF32 g) {
-  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK>;
+// EPI_BRANCH: KB sections of B (rows i * H + n), one accumulator set each, so
+// that the branches of a hidden unit meet in one thread; EPI_BRANCH_BWD: KB
+// branches in the epilogue only.
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI, int KB>
+__global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK, EPI == EPI_BRANCH ? KB : 1>::NT)
+    gemm_f32_kernel(const GemmF32 g) {
+  constexpr int SEC = EPI == EPI_BRANCH ? KB : 1;
+  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK, SEC>;
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tx = (warp % (S::TX / S::WX)) * S::WX + lane % S::WX;
@@ -122,8 +133,10 @@ __global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm
     S::A::template load<S::NT>(smem + (kb % STAGES) * S::STAGE, g.A, g.lda, m0, g.M, kb * BKT, g.K, tid);
   };
   auto load_b = [&](int kb) {
-    S::B::template load<S::NT>(smem + (kb % STAGES) * S::STAGE + S::A::FLOATS, g.B, g.ldb, n0, g.N, kb * BKT, g.K,
-                               tid);
+#pragma unroll
+    for (int i = 0; i < SEC; ++i)
+      S::B::template load<S::NT>(smem + (kb % STAGES) * S::STAGE + S::A::FLOATS + i * S::B::FLOATS,
+                                 g.B + (size_t)i * g.N * g.ldb, g.ldb, n0, g.N, kb * BKT, g.K, tid);
   };
   // Weights (b_early) were written at least two launches earlier, so their
   // first stages are fetched before the dependent-launch wait.
@@ -138,11 +151,13 @@ __global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  float acc[TM][TN];
+  float acc[SEC][TM][TN];
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+  for (int x = 0; x < SEC; ++x)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[x][i][j] = 0.f;
 
   for (int kb = 0; kb < nk; ++kb) {
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
@@ -156,15 +171,19 @@ __global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm
     const float* sb = sa + S::A::FLOATS;
 #pragma unroll
     for (int k = 0; k < BKT; k += 4) {
-      float a[4][TM], b[4][TN];
+      float a[4][TM];
       S::A::frag(sa, ty, k, a);
-      S::B::frag(sb, tx, k, b);
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int x = 0; x < SEC; ++x) {
+        float b[4][TN];
+        S::B::frag(sb + x * S::B::FLOATS, tx, k, b);
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[q][i], b[q][j], acc[i][j]);
+          for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) acc[x][i][j] = fmaf(a[q][i], b[q][j], acc[x][i][j]);
+      }
     }
   }
 #pragma unroll
@@ -175,18 +194,47 @@ __global__ void __launch_bounds__(Tile<BM, BN, TM, TN, STAGES, AK, BK>::NT) gemm
     for (int j = 0; j < TN; ++j) {
       const int n = n0 + S::B::row(tx, j);
       if (n >= g.N) continue;
-      float v = acc[i][j];
-      if (EPI >= EPI_BIAS) v += g.bias[n];
-      if (EPI == EPI_BIAS_RESID) v += g.R[(size_t)m * g.ldr + n];
-      g.C[(size_t)m * g.ldc + n] = v;
+      if (EPI == EPI_BRANCH) {  // X_i + c_i -> C, GELU of their product -> G2
+        float* c = g.C + (size_t)m * g.ldc + n;
+        float f = 1.f;
+#pragma unroll
+        for (int x = 0; x < SEC; ++x) {
+          const float v = acc[x][i][j] + g.bias[x * g.N + n];
+          c[(size_t)x * g.N] = v;
+          f = x ? f * v : v;
+        }
+        g.G2[(size_t)m * g.N + n] = gelu_f(f);
+      } else if (EPI == EPI_BRANCH_BWD) {  // the accumulator is dG; X_i are in R
+        const float* a = g.R + (size_t)m * g.ldr + n;
+        float xs[KB], f = 1.f;
+#pragma unroll
+        for (int x = 0; x < KB; ++x) {
+          xs[x] = a[(size_t)x * g.N];
+          f = x ? f * xs[x] : xs[x];
+        }
+        const float df = acc[0][i][j] * gelu_grad_f(f);
+#pragma unroll
+        for (int x = 0; x < KB; ++x) {
+          float o = 1.f;
+#pragma unroll
+          for (int l = 0; l < KB; ++l)
+            if (l != x) o *= xs[l];
+          g.C[(size_t)m * g.ldc + (size_t)x * g.N + n] = df * o;
+        }
+      } else {
+        float v = acc[0][i][j];
+        if (EPI >= EPI_BIAS) v += g.bias[n];
+        if (EPI == EPI_BIAS_RESID) v += g.R[(size_t)m * g.ldr + n];
+        g.C[(size_t)m * g.ldc + n] = v;
+      }
     }
   }
 }
 
-template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI>
+template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI, int KB = 1>
 cudaError_t launch_one(const GemmF32& g, cudaStream_t st) {
-  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK>;
-  auto k = gemm_f32_kernel<BM, BN, TM, TN, STAGES, AK, BK, EPI>;
+  using S = Tile<BM, BN, TM, TN, STAGES, AK, BK, EPI == EPI_BRANCH ? KB : 1>;
+  auto k = gemm_f32_kernel<BM, BN, TM, TN, STAGES, AK, BK, EPI, KB>;
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [&] {
@@ -204,9 +252,22 @@ cudaError_t launch_tile(const GemmF32& g, cudaStream_t st) {
     if (g.epi == EPI_BIAS) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BIAS>(g, st);
     if (g.epi == EPI_BIAS_RESID) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BIAS_RESID>(g, st);
   }
+  if (g.epi == EPI_BRANCH_BWD && g.a_kcont && !g.b_kcont) {
+    if (g.k == 1) return launch_one<BM, BN, TM, TN, STAGES, true, false, EPI_BRANCH_BWD, 1>(g, st);
+    if (g.k == 2) return launch_one<BM, BN, TM, TN, STAGES, true, false, EPI_BRANCH_BWD, 2>(g, st);
+    if (g.k == 3) return launch_one<BM, BN, TM, TN, STAGES, true, false, EPI_BRANCH_BWD, 3>(g, st);
+  }
   if (g.epi != EPI_STORE || g.b_kcont) return cudaErrorInvalidValue;
   if (g.a_kcont) return launch_one<BM, BN, TM, TN, STAGES, true, false, EPI_STORE>(g, st);
   return launch_one<BM, BN, TM, TN, STAGES, false, false, EPI_STORE>(g, st);
+}
+
+template <int BM, int BN, int TM, int TN, int STAGES>
+cudaError_t launch_branch(const GemmF32& g, cudaStream_t st) {
+  if (g.k == 1) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BRANCH, 1>(g, st);
+  if (g.k == 2) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BRANCH, 2>(g, st);
+  if (g.k == 3) return launch_one<BM, BN, TM, TN, STAGES, true, true, EPI_BRANCH, 3>(g, st);
+  return cudaErrorInvalidValue;
 }
 
 bool vec16(const float* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0; }
@@ -228,6 +289,17 @@ cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st) {
   //   1024 x 512 x 512   32x64 20.1, 64x64 22.1 (33.7) 1024 x 1024 x 2048 (weight gradient) 32x64 127.8,
   //   64x64 106.1 (189.7)
   const long long outs = (long long)g.M * g.N;
+  if (g.epi == EPI_BRANCH) {
+    // k accumulator sets a thread: smaller tiles of hidden units. 16 x 32 for the
+    // 64 MiB mix's 512 x 256 units (96 steps 63.0 ms; 32 x 32 tiles of 64 threads
+    // 65.1, separate GEMM and GELU launches 63.3); at four streams the fused
+    // launches take a small model's 512 steps from 38.1 to 36.2 ms.
+    if (!g.a_kcont || !g.b_kcont) return cudaErrorInvalidValue;
+    if (outs >= 512 << 10) return launch_branch<64, 32, 8, 4, 3>(g, st);
+    if (outs >= 24 << 10) return launch_branch<16, 32, 4, 2, 5>(g, st);
+    if (outs >= 12 << 10) return launch_branch<8, 16, 2, 2, 8>(g, st);
+    return launch_branch<8, 8, 2, 1, 8>(g, st);
+  }
   if (outs >= 1 << 20) return launch_tile<64, 64, 8, 4, 3>(g, st);
   if (outs >= 192 << 10) return launch_tile<32, 64, 4, 4, 4>(g, st);
   if (outs >= 96 << 10) return launch_tile<16, 32, 4, 2, 6>(g, st);

@@ -138,61 +138,6 @@ cudaError_t launch_ln_fwd(const float* X, const float* g, const float* be, float
 }
 
 // ============================================================================================
-// MBRB branch fusion (Eqs. 11-12): G = GELU(X_1 * ... * X_k), exact erf GELU.
-// ============================================================================================
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float x) {
-  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
-__global__ void branch_gelu_kernel(const float* __restrict__ A, int b, int H, int k, float* __restrict__ G) {
-  pdl_wait();
-  pdl_launch();
-  const size_t n = (size_t)b * H;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    size_t r = e / H, h = e - r * H;
-    const float* a = A + r * (size_t)k * H + h;
-    float f = a[0];
-    for (int i = 1; i < k; ++i) f *= a[(size_t)i * H];
-    G[e] = gelu_f(f);
-  }
-}
-
-cudaError_t launch_branch_gelu(const float* A, int b, int H, int k, float* G, cudaStream_t st) {
-  size_t n = (size_t)b * H;
-  int grid = (int)((n + 255) / 256);
-  return launch_k(branch_gelu_kernel, dim3(grid), dim3(256), 0, st, A, b, H, k, G);
-}
-
-__global__ void branch_gelu_bwd_kernel(const float* __restrict__ dG, const float* __restrict__ A, int b, int H,
-                                       int k, float* __restrict__ dA) {
-  pdl_wait();
-  pdl_launch();
-  const size_t n = (size_t)b * H;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    size_t r = e / H, h = e - r * H;
-    const float* a = A + r * (size_t)k * H + h;
-    float* da = dA + r * (size_t)k * H + h;
-    float f = a[0];
-    for (int i = 1; i < k; ++i) f *= a[(size_t)i * H];
-    float df = dG[e] * gelu_grad_f(f);
-    for (int i = 0; i < k; ++i) {
-      float o = 1.0f;
-      for (int l = 0; l < k; ++l)
-        if (l != i) o *= a[(size_t)l * H];
-      da[(size_t)i * H] = df * o;
-    }
-  }
-}
-
-cudaError_t launch_branch_gelu_bwd(const float* dG, const float* A, int b, int H, int k, float* dA,
-                                   cudaStream_t st) {
-  size_t n = (size_t)b * H;
-  int grid = (int)((n + 255) / 256);
-  return launch_k(branch_gelu_bwd_kernel, dim3(grid), dim3(256), 0, st, dG, A, b, H, k, dA);
-}
-
-// ============================================================================================
 // Column sums over rows of the FP32 path (bias and LN-affine gradients), all of
 // a block's tensors in one launch, fixed order: warp w sums rows w, w+8, ...
 // for 32 columns; then warps are added in order.

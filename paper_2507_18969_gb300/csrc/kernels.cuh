@@ -23,8 +23,6 @@ cudaError_t launch_embed(const uint8_t* data, Split sp, const StepCtl* ctl, cons
 // Row-wise LayerNorm: xhat, rstd, X0 = g * xhat + beta.
 cudaError_t launch_ln_fwd(const float* X, const float* g, const float* be, float* xhat, float* rstd,
                           float* X0, int b, int F, cudaStream_t st);
-// G = GELU(prod_i A[:, iH:(i+1)H]).
-cudaError_t launch_branch_gelu(const float* A, int b, int H, int k, float* G, cudaStream_t st);
 // Which streams of a step are active: `active` (model API) if set, else
 // the stream still has bytes at time index ctl->i. ctl == nullptr: all.
 struct FdmAct {
@@ -70,8 +68,6 @@ struct HeadArgs {
 cudaError_t launch_head(const HeadArgs& a, cudaStream_t st);
 
 // ---- backward -----------------------------------------------------------------------------
-cudaError_t launch_branch_gelu_bwd(const float* dG, const float* A, int b, int H, int k, float* dA,
-                                   cudaStream_t st);
 // out[c] = sum_r X[r][c] (or sum_r X[r][c] * Y[r][c] when Y != nullptr) for each
 // job, fixed order (the chunk fields of jobs unused).
 struct ColsumJobs;
@@ -206,7 +202,11 @@ cudaError_t launch_cdf_quantize(const float* p, int rows, uint32_t* freq, uint32
 // ---- GEMM (FP32 SIMT) ------------------------------------------------------------------------
 // C[m][n] = sum_k A(m,k) B(n,k) (+ bias[n]) (+ R[m][n]).
 // A(m,k) = a_kcont ? A[m*lda + k] : A[k*lda + m];  B(n,k) = b_kcont ? B[n*ldb + k] : B[k*ldb + n].
-enum Epi { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_RESID = 2 };
+// EPI_BRANCH (Eqs. 10-12; both k-contiguous): N hidden units, B holds k sections
+// of N rows; C[m][i*N + n] = X_i = acc_i + bias[i*N + n], G2[m][n] = GELU(prod X_i).
+// EPI_BRANCH_BWD (B not k-contiguous): acc = dG, R[m][i*N + n] = X_i,
+// C[m][i*N + n] = dG GELU'(prod X) prod_{l != i} X_l.
+enum Epi { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_RESID = 2, EPI_BRANCH = 3, EPI_BRANCH_BWD = 4 };
 struct GemmF32 {
   int M, N, K;
   const float* A; int lda; bool a_kcont;
@@ -215,7 +215,9 @@ struct GemmF32 {
   int epi;
   const float* bias;
   const float* R; int ldr;
-  bool b_early;  // B was written at least two launches before (weights): fetched ahead of the PDL wait
+  int k = 1;         // branches (EPI_BRANCH, EPI_BRANCH_BWD)
+  float* G2 = nullptr;
+  bool b_early = false;  // B was written at least two launches before (weights): fetched ahead of the PDL wait
 };
 cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st);
 
