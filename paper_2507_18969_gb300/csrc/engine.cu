@@ -14,9 +14,9 @@
 //   FP32  SIMT GEMMs and separate element-wise kernels.
 //   BF16  tcgen05 GEMMs whose epilogues fuse the MBRB element-wise ops and
 //         write the BF16 (and transposed BF16) operands of the next GEMMs; the
-//         weight-gradient GEMMs and column sums, which nothing on the step's
-//         critical path waits for, run on a side stream forked per layer and
-//         joined before Adam.
+//         weight-gradient GEMMs (first side stream) and the column sums and
+//         each layer's Adam (second), which nothing on the step's critical path
+//         waits for, are forked per layer and joined at the step's end.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -1670,16 +1670,13 @@ int Model::step_delayed(const StepIO& io, cudaStream_t st) {
 }
 
 int Model::launches_per_step() const {
-  if (precision != EDPC_FP32) {
-    // forward: embed (with block 0's LN) + 3 per block (2 for block 0) + LTE (2 GEMMs + FDM) + head GEMM + head
-    int n = 1 + 3 * d.n - (d.nloc > 0 ? 1 : 0) + 3 + 1 + 1;
-    // backward: head dW/colsum/dX, per block 3 main + 3 side, LTE 3 + 2 side ... + embed
-    n += 3 + 6 * d.n + 3 + 4 + 1;
-    return n + 3;  // adam, transpose, advance
-  }
-  int n = 1 + 4 * d.n + 3 + 1 + 1;
-  n += 3 + 10 * d.n + 3 + 1 + 3 + 1;
-  return n + 2;
+  const bool bf16 = precision != EDPC_FP32;
+  // forward: embedding, 3 per block (BF16: block 0's LN with the embedding), LTE (2 GEMMs + FDM), head GEMM, head
+  int n = 1 + 3 * d.n - (bf16 && d.nloc > 0 ? 1 : 0) + 3 + 2;
+  // backward: head dW / column sum / dX, per block 3 main + 3 side, LTE 2 + FDM + 4 side, embedding
+  n += 3 + 6 * d.n + 7 + 1;
+  // Adam: one per layer; delayed update: one, the transposed copies and the step control
+  return n + (delayed ? 2 + (bf16 ? 1 : 0) : d.n + 2);
 }
 
 }  // namespace edpc

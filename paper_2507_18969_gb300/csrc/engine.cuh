@@ -52,7 +52,7 @@ class Model {
   float *dY = nullptr, *dXp = nullptr;
   float* emb_part = nullptr;              // embedding-adjoint chunk partials (many positions)
   unsigned* emb_cnt = nullptr;            // their arrival counters, one per byte value
-  float* cs_part = nullptr;               // column-sum chunk partials (side stream)
+  float* cs_part = nullptr;               // column-sum chunk partials (second side stream)
   unsigned* cs_cnt = nullptr;             // column-sum arrival counters, one per 32-column tile
   int cs_tiles = 0;                       // tiles cs_cnt is sized for
   int cs_cols = 0;                        // tile columns (per chunk) cs_part is sized for
@@ -244,7 +244,7 @@ class Model {
   int colsums(ColsumJobs cj, cudaStream_t st);  // column sums with the model's chunk scratch
   int fdm_fwd_call(const StepIO& io, cudaStream_t st);
   int fdm_bwd_call(const StepIO& io, cudaStream_t st);
-  int fdm_bwd_joined(const StepIO& io, cudaStream_t st);  // waits for the side stream from 2048 streams on
+  int fdm_bwd_joined(const StepIO& io, cudaStream_t st);  // waits for the side streams from 2048 streams on
   int build_tc_plan_one();
   void save_parity(int q);                                 // parity q <- the members
   const TcPlan& plan() const { return delayed ? par[cur].tcp : tcp; }

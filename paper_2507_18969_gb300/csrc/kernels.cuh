@@ -222,8 +222,8 @@ struct GemmF32 {
 cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st);
 
 // ---- BF16 path: fused operand production -----------------------------------------------------
-// Rows are processed 16 per CTA so that the transposed copy YT[c][r] (ld ldT, a
-// multiple of 16; padding rows are written as zero) goes out in 32-byte runs.
+// The transposed copies YT[c][r] have a leading dimension ldT that is a multiple
+// of kRowsT (padding rows are written as zero), so that runs of rows are aligned.
 constexpr int kRowsT = 16;
 // LayerNorm forward writing xhat, rstd and the BF16 copies of X0 (row-major and transposed).
 // Grouped mode (rg != nullptr): row r uses g + rg[r] * gs and be + rg[r] * gs.

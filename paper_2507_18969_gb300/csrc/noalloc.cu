@@ -1,13 +1,14 @@
 // Range encoding without any device allocation.
 //
-// edpc_range_encode obtains its per-call scratch (one coder state, output
-// offset and capacity per stream) from cudaMalloc and releases it with
-// cudaFree. Some callers cannot allow that: services that reserve their whole
-// device-memory budget at start-up and refuse later allocations, and
+// edpc_range_encode keeps a stream's coder state in registers from the first
+// symbol to the flush. This entry point codes through the session's kernels
+// instead (a prefix, coding and flush launch over coder states in memory), for
+// callers that may not allocate device memory: services that reserve their
+// whole device-memory budget at start-up and refuse later allocations, and
 // latency-sensitive loops that cannot absorb the device-wide synchronisation
-// cudaFree may perform. For them, edpc_range_encode_noalloc keeps the scratch
-// in a fixed array that is part of the library image itself: it exists on
-// every GPU that loads the library, from load until process exit.
+// cudaFree may perform. The states, output offsets and capacities are a fixed
+// array that is part of the library image itself: it exists on every GPU that
+// loads the library, from load until process exit.
 #include <mutex>
 
 #include "kernels.cuh"
