@@ -1404,6 +1404,7 @@ EmbAdam Model::emb_adam(const StepIO& io) const {
 }
 
 int Model::forward_bf16(const StepIO& io, cudaStream_t st) {
+  nfork_ = 0;  // the waits on the previous pass's forks have all been issued; a forward pass may be repeated alone
   const bool f8m = precision == EDPC_FP8E4M3;
   if (f8m) {
     std::fill(f8_done.begin(), f8_done.end(), 0);
@@ -1467,7 +1468,7 @@ int Model::fdm_bwd_joined(const StepIO& io, cudaStream_t st) {
 
 int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
   const int kH = d.k * d.H;
-  nfork_ = 0;  // (FP8's fork in the forward pass has its event waited for by then)
+  nfork_ = 0;  // (so has the wait on the forward pass's fork)
   const bool f8m = precision == EDPC_FP8E4M3;
   // the dX GEMMs read FP8's transposed shadows (delayed update: made during the previous step)
   if (f8m && !delayed) EDPC_CUDA(cudaStreamWaitEvent(st, tr_ev, 0));
