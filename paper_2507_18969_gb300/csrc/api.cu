@@ -439,14 +439,20 @@ struct edpc_session {
   // (x_chunk: `chunk` steps, instantiated twice with separate events and
   // launched alternately; x_one_t: one step) are made when profiling is first
   // turned on.
-  // run_steps: instantiating and destroying a graph takes time in proportion
-  // to its nodes (about 60 a step). 16 steps instead of 64, instantiated once
-  // instead of twice, took opening and closing a session of the 64 MiB mix's
-  // model from 26 to 6 ms. Schedules that keep an FDM update running under the
-  // next step's layers join it at a graph's end, so they keep `chunk` steps.
+  // run_steps and run_min: capturing, instantiating and destroying a graph takes
+  // time in proportion to its nodes (about 60 a step), and all that the longer
+  // graph saves is 1 to 2.5 us a step of hand-over between launches. So x_run
+  // is made for sessions of run_min steps and more only. Whole compressions, one-step
+  // graph alone / with the 8-step graph / with a 16-step one, in ms:
+  //   default model, FP32, 4 streams     24 steps 2.3 / 3.5 / 4.8     512: 36.2 / 36.0 / 37.1   2048: 142.0 / 137.2 / 138.9
+  //   64 MiB mix's model, 512 streams    24 steps 8.7 / 10.5 / 12.7  1024: 313.8 / 314.4 / 316.9  2048: 628.5 / 625.9 / 628.4
+  //   1 GiB mix's model, 16 streams      24 steps 8.8 / 11.3 / 13.9  1024: 307.6 / 307.4 / 310.8  2048: 611.9 / 609.9 / 613.1
+  // They meet at 500 steps (small models) to 1700 (64 MiB mix, 64 streams).
+  // Schedules that keep an FDM update running under the next step's layers join
+  // it at a graph's end, so they have `chunk` steps a graph, from as many steps on.
   cudaGraph_t g_run = nullptr, g_one = nullptr, g_chunk = nullptr, g_one_t = nullptr;
   cudaGraphExec_t x_run = nullptr, x_one = nullptr, x_chunk[2] = {}, x_one_t = nullptr;
-  static constexpr int kRunSteps = 16;
+  static constexpr int kRunSteps = 8, kRunMin = 1024;
   int run_steps = kRunSteps;
   int graph_kernels = 0;  // kernels per step
 
@@ -618,7 +624,7 @@ int edpc_session::capture_graph() {
     EDPC_CUDA(cudaGraphNodeGetType(nd, &t));
     if (t == cudaGraphNodeTypeKernel) ++graph_kernels;
   }
-  if (steps_total < (uint64_t)run_steps) return EDPC_OK;
+  if (steps_total < (uint64_t)(model.side_fdm ? kChunk : kRunMin)) return EDPC_OK;
   EDPC_TRY(capture(run_steps, -1, &g_run));
   EDPC_CUDA(cudaGraphInstantiate(&x_run, g_run, 0));
   return EDPC_OK;
