@@ -1483,7 +1483,9 @@ int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
     EDPC_TRY(colsums(cj, side2));
   }
   {
-    PdlScope scope(!f8m);  // FP8: the stream also waits on the shadows' event
+    // FP8: the stream also waits on the shadows' event; delayed update: this is
+    // the first launch after bwd_st's wait for the step's start
+    PdlScope scope(!f8m && !delayed);
     EDPC_TRY(run_tc(kSiteHeadDx, st));  // dOut of the last block
   }
   EDPC_TRY(adam_layer(io, d.n + 1, st));
