@@ -14,8 +14,6 @@
 #include "kernels.cuh"
 #include "launch.cuh"
 
-#include <mutex>
-
 namespace edpc {
 
 namespace {
@@ -235,11 +233,9 @@ template <int BM, int BN, int TM, int TN, int STAGES, bool AK, bool BK, int EPI,
 cudaError_t launch_one(const GemmF32& g, cudaStream_t st) {
   using S = Tile<BM, BN, TM, TN, STAGES, AK, BK, EPI == EPI_BRANCH ? KB : 1>;
   auto k = gemm_f32_kernel<BM, BN, TM, TN, STAGES, AK, BK, EPI, KB>;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [&] {
-    attr = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
-  });
+  static OncePerDevice once;
+  const cudaError_t attr = once_on_device(
+      once, [&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem); });
   if (attr != cudaSuccess) return attr;
   return launch_k(k, dim3(div_up(g.N, BN), div_up(g.M, BM)), dim3(S::NT), S::kSmem, st, g);
 }

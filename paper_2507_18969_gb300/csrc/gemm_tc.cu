@@ -242,12 +242,12 @@ __global__ void __launch_bounds__(kTcThreads, MODE == TC_PLAIN || BN > 64 ? 2 : 
 template <int BN, int MODE, int KB, bool F8, bool GR>
 cudaError_t launch_bn_mode_g(const TcGemm& g, cudaStream_t st) {
   auto k = gemm_tc_kernel<BN, MODE, KB, F8, GR>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<BN>());
-    if (attr_err == cudaSuccess)
-      attr_err = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  static OncePerDevice once;
+  const cudaError_t attr_err = once_on_device(once, [&] {
+    const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<BN>());
+    return r != cudaSuccess
+               ? r
+               : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   });
   if (attr_err != cudaSuccess) return attr_err;
   TcEpi e{g.M, g.N, g.K, g.H, g.k, g.C, g.ldc, g.Cb, g.ldcb, g.CbT, g.ldct, g.bias, g.R, g.ldr, g.Aux, g.ldaux, g.err,

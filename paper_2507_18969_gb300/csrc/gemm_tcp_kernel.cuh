@@ -23,7 +23,6 @@
 #include <cudaTypedefs.h>
 
 #include <climits>
-#include <mutex>
 
 #include "gemm_tc.cuh"
 #include "gemm_tc_dev.cuh"
@@ -220,23 +219,21 @@ __global__ void __launch_bounds__(192, 1)
   }
 }
 
-int sm_count();
-
 template <int BN, int MODE, int KB, bool F8>
 cudaError_t launch_p(const TcGemm& g, cudaStream_t st) {
   auto k = gemm_tcp_kernel<BN, MODE, KB, F8>;
   constexpr int SW = (MODE == TC_BRANCH) ? BN / KB : BN;
   // the tensor map's box must be one section of B
   if (g.box_b != SW) return cudaErrorInvalidValue;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  static int max_ctas = 0;
-  std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem_bytes<BN>());
-    if (attr_err == cudaSuccess)
-      attr_err = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    max_ctas = sm_count();
+  static OncePerDevice once;
+  cudaError_t attr_err = once_on_device(once, [&] {
+    const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem_bytes<BN>());
+    return r != cudaSuccess
+               ? r
+               : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   });
+  int max_ctas = 0;
+  if (attr_err == cudaSuccess) attr_err = sm_count(&max_ctas);
   if (attr_err != cudaSuccess) return attr_err;
   const int ntn = (MODE == TC_BRANCH) ? (g.H + SW - 1) / SW : (g.N + BN - 1) / BN;
   const int ntm = (g.M + BM - 1) / BM;

@@ -31,8 +31,6 @@
 //                      of half w >> 2; loads that do not depend on the
 //                      accumulator, and GELU's derivative, come before.
 // Waits are bounded as in gemm_tc_kernel.
-#include <mutex>
-
 #include "gemm_tc.cuh"
 #include "gemm_tc_dev.cuh"
 #include "kernels.cuh"
@@ -324,13 +322,13 @@ __global__ void __launch_bounds__(kThreadsS, 1)
 template <int NS, int MODE, int KB>
 cudaError_t launch_s(const TcGemm& g, cudaStream_t st) {
   auto k = gemm_tcs_kernel<NS, MODE, KB>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem_bytes_s<NS>(kStagesS));
-    if (attr_err == cudaSuccess)
-      attr_err = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  static OncePerDevice once;
+  const cudaError_t attr_err = once_on_device(once, [&] {
+    const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem_bytes_s<NS>(kStagesS));
+    return r != cudaSuccess
+               ? r
+               : cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   });
   if (attr_err != cudaSuccess) return attr_err;
   TcEpi e{};

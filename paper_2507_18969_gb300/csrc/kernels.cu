@@ -8,8 +8,6 @@
 
 #include <algorithm>
 
-#include <mutex>
-
 #include "kernels.cuh"
 #include "launch.cuh"
 
@@ -418,17 +416,14 @@ template <int FP>
 cudaError_t launch_fdm_fwd_persist(const float* Xp, const float* U, float* Y, int b, __nv_bfloat16* Yb,
                                    __nv_bfloat16* YbT, int ldT, int* err, const FdmAct& act, cudaStream_t st) {
   const size_t smem = (size_t)kFdmPersistRing * 16384 + (size_t)FP * 4 + 64 + 64;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  static int grid = 0;
-  std::call_once(once, [&] {
-    attr = cudaFuncSetAttribute(fdm_fwd_persist_kernel<FP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int dev = 0, sms = 0;
-    if (attr == cudaSuccess) attr = cudaGetDevice(&dev);
-    if (attr == cudaSuccess) attr = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    grid = sms * kFdmPersistPerSm;
+  static OncePerDevice once;
+  cudaError_t attr = once_on_device(once, [&] {
+    return cudaFuncSetAttribute(fdm_fwd_persist_kernel<FP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
+  int sms = 0;
+  if (attr == cudaSuccess) attr = sm_count(&sms);
   if (attr != cudaSuccess) return attr;
+  const int grid = sms * kFdmPersistPerSm;
   const int g = b < grid ? b : grid;
   return launch_k(fdm_fwd_persist_kernel<FP>, dim3(g), dim3(FdmRing<FP>::NT), smem, st, Xp, U, Y, Yb, YbT, ldT, err,
                   act, b);
@@ -843,18 +838,16 @@ cudaError_t launch_fdm_dx(const FdmSplitArgs& a, cudaStream_t st) {
 
 template <int NCH>
 cudaError_t launch_adam_persist(const FdmSplitArgs& a, cudaStream_t st) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    // The CTA stays resident for the whole update: keep its SM configured for
-    // the largest shared-memory carveout, so GEMM CTAs still fit beside it.
-    e = cudaFuncSetAttribute(fdm_adam_persist_kernel<NCH>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-  }
+  // The CTA stays resident for the whole update: keep its SM configured for
+  // the largest shared-memory carveout, so GEMM CTAs still fit beside it.
+  static OncePerDevice once;
+  cudaError_t e = once_on_device(once, [] {
+    return cudaFuncSetAttribute(fdm_adam_persist_kernel<NCH>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                cudaSharedmemCarveoutMaxShared);
+  });
+  int sms = 0;
+  if (e == cudaSuccess) e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
   return launch_k(fdm_adam_persist_kernel<NCH>, dim3(sms), dim3(32 * kAdamWarps), 0, st, a);
 }
 
@@ -1095,10 +1088,9 @@ template <int DT, class Scratch, class... A>
 static cudaError_t launch_emb_owner(dim3 grid, cudaStream_t st, A... args) {
   constexpr size_t smem = 8 * sizeof(Scratch);
   auto k = embed_bwd_owner_kernel<DT, Scratch>;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once,
-                 [&] { attr = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+  static OncePerDevice once;
+  const cudaError_t attr = once_on_device(
+      once, [&] { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
   if (attr != cudaSuccess) return attr;
   return launch_k(k, grid, dim3(256), smem, st, args...);
 }
@@ -1164,10 +1156,9 @@ __global__ void __launch_bounds__(256) embed_bwd_groups_kernel(const uint8_t* __
 template <int DT, class... A>
 static cudaError_t launch_emb_groups(dim3 grid, cudaStream_t st, A... args) {
   constexpr size_t smem = 8 * sizeof(EmbWide);
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(embed_bwd_groups_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static OncePerDevice once;
+  const cudaError_t attr = once_on_device(once, [] {
+    return cudaFuncSetAttribute(embed_bwd_groups_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (attr != cudaSuccess) return attr;
   return launch_k(embed_bwd_groups_kernel<DT>, grid, dim3(256), smem, st, args...);

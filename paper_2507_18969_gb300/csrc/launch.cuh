@@ -12,7 +12,25 @@
 
 #include <utility>
 
+#include "once.cuh"
+
 namespace edpc {
+
+// f (kernel attributes, ...) once on the current device.
+template <class F>
+inline cudaError_t once_on_device(OncePerDevice& once, F&& f) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : once.run(dev, f);
+}
+
+// The current device's SM count (at least 1).
+inline cudaError_t sm_count(int* n) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+  return e;
+}
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -295,14 +295,15 @@ extern "C" int edpc_ksg_mi(const float* Z, const float* Y, uint32_t N, uint32_t 
   if (dz < 1 || dy < 1 || dz + dy > 8192) return fail(EDPC_EINVAL, "dz, dy >= 1 and dz + dy <= 8192");
   constexpr size_t kDistSmem = (size_t)kStages * 2 * kTile * kLd * sizeof(float);
   constexpr size_t kListSmem = 128 * 1024;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(ksg_dist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(ksg_dist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(ksg_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem);
+  static OncePerDevice once;
+  const cudaError_t attr = once_on_device(once, [] {
+    cudaError_t r =
+        cudaFuncSetAttribute(ksg_dist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(ksg_dist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(ksg_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem);
+    return r;
   });
   if (attr != cudaSuccess) return fail(EDPC_ECUDA, std::string("ksg attribute: ") + cudaGetErrorString(attr));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
