@@ -18,8 +18,6 @@
 // psi(k) + psi(N) - mean(psi(c_z + 1) + psi(c_y + 1)) in FP64.
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -227,44 +225,38 @@ __global__ void ksg_select_kernel(const float* __restrict__ D, int R, int ld, in
 // The distance workspace comes from a memory pool of the library's own, one per
 // device, that keeps at most kWorkspace bytes between calls (stream-ordered, so
 // concurrent calls on any threads and streams get buffers of their own; what
-// they hold beyond that goes back to the device when they synchronize).
+// they hold beyond that goes back to the device when they synchronize). A pool
+// lives as long as its device's context: nothing destroys it at process exit,
+// when the driver may be gone already, and a process that resets a device with
+// cudaDeviceReset must not call this entry point on it again.
 constexpr size_t kWorkspace = (size_t)64 << 20;
-
-struct WorkspacePools {
-  std::mutex mu;
-  std::map<int, cudaMemPool_t> pool;
-  ~WorkspacePools() {
-    for (auto& p : pool) cudaMemPoolDestroy(p.second);
-  }
-};
+cudaMemPool_t g_pool[OncePerDevice::kDevices] = {};
 
 cudaError_t workspace_alloc(float** p, size_t bytes, cudaStream_t st) {
-  static WorkspacePools pools;
+  static OncePerDevice once;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  cudaMemPool_t pool = nullptr;
-  {
-    std::lock_guard<std::mutex> lock(pools.mu);
-    auto it = pools.pool.find(dev);
-    if (it == pools.pool.end()) {
-      cudaMemPoolProps props{};
-      props.allocType = cudaMemAllocationTypePinned;
-      props.handleTypes = cudaMemHandleTypeNone;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
-      uint64_t keep = kWorkspace;
-      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-      if (e != cudaSuccess) {
-        cudaMemPoolDestroy(pool);
-        return e;
-      }
-      it = pools.pool.emplace(dev, pool).first;
-    }
-    pool = it->second;
-  }
-  return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, pool, st);
+  if (dev >= OncePerDevice::kDevices)  // the device's default pool, which keeps nothing unless it is told to
+    return cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st);
+  e = once.run(dev, [&] {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t r = cudaMemPoolCreate(&pool, &props);
+    if (r != cudaSuccess) return r;
+    uint64_t keep = kWorkspace;
+    r = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (r != cudaSuccess)
+      cudaMemPoolDestroy(pool);
+    else
+      g_pool[dev] = pool;
+    return r;
+  });
+  return e != cudaSuccess ? e : cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool[dev], st);
 }
 
 // psi(x) for x >= 1: recurrence up to x >= 10, then the asymptotic series
