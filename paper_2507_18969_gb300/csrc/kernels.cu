@@ -1296,18 +1296,24 @@ struct EncIO {
 };
 
 // n bytes of v into the window from pos on, after a carry into the bytes before
-// them (done unless err). Returns the new position, and err in the upper half:
-// bytes beyond the capacity set it. By value, so that the state stays in registers.
+// them. Returns the new position, and err in the upper half: bytes beyond the
+// capacity are lost and set it, to kLostFF while every lost byte is 0xFF (a carry
+// goes through those into the window, once), else to kLost. By value, so that the
+// state stays in registers.
+constexpr uint32_t kLost = 1, kLostFF = 2;
 __device__ __noinline__ unsigned long long enc_put_slow(uint8_t* out, uint32_t cap, uint32_t pos, uint32_t err, uint32_t v,
                                                         uint32_t n, bool carry) {
-  if (carry && !err)
+  if (carry && err != kLost) {
     for (uint32_t p = pos; p-- > 0;)
       if (++out[p] != 0) break;
+    if (err) err = kLost;
+  }
   for (uint32_t k = n; k-- > 0;) {
+    const uint8_t byte = (uint8_t)(v >> (8 * k));
     if (pos < cap)
-      out[pos++] = (uint8_t)(v >> (8 * k));
+      out[pos++] = byte;
     else
-      err = 1;
+      err = err != kLost && byte == 0xFF ? kLostFF : kLost;
   }
   return (unsigned long long)err << 32 | pos;
 }
