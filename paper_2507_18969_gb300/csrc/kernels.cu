@@ -466,6 +466,18 @@ __device__ __forceinline__ void adam1(float& p, float& m, float& v, float g, flo
   p = p - lr * mh / (sqrtf(vh) + kAdamEps);
 }
 
+// adam1 with the contractions spelled out as the compiler chooses them in the fused
+// adjoint (fdm_bwd_kernel<1> and the generic one: G; the wider ones: not G). The
+// update that runs on its own stream instead (EDPC_FLAG_OVERLAP_FDM) must give the
+// same bits, since the container is decoded by the fused one; left to the compiler
+// its kernels contracted other products than the fused ones at most widths.
+template <bool G>
+__device__ __forceinline__ void adam1_fused(float& p, float& m, float& v, float g, float lr, float bc1, float bc2) {
+  m = G ? __fmaf_rn(1.0f - kB1, g, __fmul_rn(kB1, m)) : __fmaf_rn(kB1, m, __fmul_rn(1.0f - kB1, g));
+  v = __fmaf_rn(__fmul_rn(1.0f - kB2, g), g, __fmul_rn(kB2, v));
+  p = p - lr * (m / bc1) / (sqrtf(v / bc2) + kAdamEps);
+}
+
 __device__ __forceinline__ void store_dxp(const FdmBwdArgs& a, int s, int i, float v) {
   a.dXp[(size_t)s * a.Fp + i] = v;
   if (a.dXpb) a.dXpb[(size_t)s * a.Fp + i] = __float2bfloat16_rn(v);
@@ -700,10 +712,10 @@ __global__ void __maxnreg__(80) fdm_adam_persist_kernel(FdmSplitArgs a) {
 #pragma unroll
         for (int q = 0; q < NU; ++q) {
           const float4 dy = reinterpret_cast<const float4*>(a.dy_pend + dyo[h])[lane + 32 * q];
-          adam1(u[h][q].x, m[h][q].x, v[h][q].x, xi[h] * dy.x, pd.lr, pd.bc1, pd.bc2);
-          adam1(u[h][q].y, m[h][q].y, v[h][q].y, xi[h] * dy.y, pd.lr, pd.bc1, pd.bc2);
-          adam1(u[h][q].z, m[h][q].z, v[h][q].z, xi[h] * dy.z, pd.lr, pd.bc1, pd.bc2);
-          adam1(u[h][q].w, m[h][q].w, v[h][q].w, xi[h] * dy.w, pd.lr, pd.bc1, pd.bc2);
+          adam1_fused<NCH == 1>(u[h][q].x, m[h][q].x, v[h][q].x, xi[h] * dy.x, pd.lr, pd.bc1, pd.bc2);
+          adam1_fused<NCH == 1>(u[h][q].y, m[h][q].y, v[h][q].y, xi[h] * dy.y, pd.lr, pd.bc1, pd.bc2);
+          adam1_fused<NCH == 1>(u[h][q].z, m[h][q].z, v[h][q].z, xi[h] * dy.z, pd.lr, pd.bc1, pd.bc2);
+          adam1_fused<NCH == 1>(u[h][q].w, m[h][q].w, v[h][q].w, xi[h] * dy.w, pd.lr, pd.bc1, pd.bc2);
           __stcs(reinterpret_cast<float4*>(a.U + base[h]) + lane + 32 * q, u[h][q]);
           __stcs(reinterpret_cast<float4*>(a.Um + base[h]) + lane + 32 * q, m[h][q]);
           __stcs(reinterpret_cast<float4*>(a.Uv + base[h]) + lane + 32 * q, v[h][q]);
@@ -799,6 +811,8 @@ __global__ void __launch_bounds__(256) fdm_dx_generic_kernel(FdmSplitArgs a) {
   }
 }
 
+// FUSED: the overlapped update of Algorithm 1's schedule; else the delayed update's.
+template <bool FUSED>
 __global__ void __launch_bounds__(256) fdm_adam_generic_kernel(FdmSplitArgs a) {
   pdl_wait();
   pdl_launch();
@@ -816,7 +830,11 @@ __global__ void __launch_bounds__(256) fdm_adam_generic_kernel(FdmSplitArgs a) {
     const float* src = a.Ub ? a.Ub : a.U;
     for (int j = lane; j < Fp; j += 32) {
       float u = src[ro + j], m = a.Um[ro + j], v = a.Uv[ro + j];
-      adam1(u, m, v, xi * a.dy_pend[(size_t)s * Fp + j], pd.lr, pd.bc1, pd.bc2);
+      const float g = xi * a.dy_pend[(size_t)s * Fp + j];
+      if (FUSED)
+        adam1_fused<true>(u, m, v, g, pd.lr, pd.bc1, pd.bc2);
+      else
+        adam1(u, m, v, g, pd.lr, pd.bc1, pd.bc2);
       a.U[ro + j] = u;
       a.Um[ro + j] = m;
       a.Uv[ro + j] = v;
@@ -867,7 +885,9 @@ cudaError_t launch_fdm_adam(const FdmSplitArgs& a, cudaStream_t st, bool persist
     case 384: return launch_k(fdm_adam_kernel<3>, grid, dim3(256), 0, st, a);
     case 512: return launch_k(fdm_adam_kernel<4>, grid, dim3(256), 0, st, a);
     case 1024: return launch_k(fdm_adam_kernel<8>, grid, dim3(256), 0, st, a);
-    default: return launch_k(fdm_adam_generic_kernel, grid, dim3(256), 0, st, a);
+    default:
+      return launch_k(persistent ? fdm_adam_generic_kernel<true> : fdm_adam_generic_kernel<false>, grid, dim3(256), 0,
+                      st, a);
   }
 }
 
