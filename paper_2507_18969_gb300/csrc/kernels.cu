@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(256) fdm_adam_kernel(FdmSplitArgs a) {
 // Persistent form of the update, built to run beside the step's other kernels:
 // one CTA of 512 threads per SM, at most 80 registers a thread and no shared
 // memory, so the step's tensor-core GEMM CTAs still fit on every SM. The FDM
-// rows are cut into units of 32 lanes x NU float4 (NU = min(NCH, 2)); warp w of
+// rows are cut into units of 32 lanes x NU float4 (2, or 1 for odd NCH); warp w of
 // CTA c owns units u = c * 16 + w, u + W, u + 2W, ... (W = 16 * grid) and
 // updates two units per iteration, so every lane has 6 NU independent
 // 16-byte loads in flight. Warps never synchronise.
@@ -670,7 +670,7 @@ constexpr int kAdamWarps = 16;
 template <int NCH>
 __global__ void __maxnreg__(80) fdm_adam_persist_kernel(FdmSplitArgs a) {
   constexpr int FP = 128 * NCH;
-  constexpr int NU = NCH < 2 ? NCH : 2;  // float4 per lane per unit
+  constexpr int NU = NCH % 2 ? 1 : 2;    // float4 per lane per unit
   constexpr int UPR = NCH / NU;          // units per FDM row
   pdl_wait();
   pdl_launch();

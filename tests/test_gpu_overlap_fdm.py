@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", [edpc.EDPC_BF16, edpc.EDPC_FP8E4M3])
-@pytest.mark.parametrize("latent", [0, 8, 72, 128, 200, 256, 512, 1024])  # 0: the FDM is F x F, F = 128
+@pytest.mark.parametrize("latent", [0, 8, 72, 128, 200, 256, 384, 512, 1024])  # 0: the FDM is F x F, F = 128
 def test_overlapped_update_codes_the_same_container(prec, latent):
     b, steps = (40, 100) if latent <= 256 else (12, 70)
     kw = dict(streams=b, precision=prec, context=8, embed_dim=16, latent=latent, hidden=64, blocks=2, branches=2, seed=3)
