@@ -397,9 +397,9 @@ int edpc_range_encode(const uint32_t* sym, uint32_t nsym, uint32_t streams, uint
 
 /*
  * The paper has no counterpart to this entry point; it serves callers that
- * cannot allocate device memory per call, such as services that reserve
- * their whole GPU memory budget at start-up and refuse later allocations, or
- * loops that cannot absorb the device-wide synchronisation cudaFree may do.
+ * cannot allocate per call at all. (edpc_range_encode makes no device
+ * allocation either, but holds the streams' lengths in a host buffer; it needs
+ * one launch instead of five and has none of the limits below.)
  *
  * Same arguments, layout and result as edpc_range_encode, but the per-stream
  * coder state, output offsets and capacities live in a fixed scratch array

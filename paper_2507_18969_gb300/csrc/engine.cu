@@ -794,8 +794,8 @@ int Model::fp8_shadow(const void* src, int rows, int cols, int ld) {
   sh.cols = cols;
   sh.ld = ld;
   sh.ld8 = (int)round_up(cols, 16);
-  // quantized columns: whole 8-element vectors; a transposed operand's extra
-  // columns up to ld are its zero padding (b rounded up to 16)
+  // quantized columns: whole 8-element vectors; a transposed operand has up to
+  // seven columns beyond b (see kRowsT)
   sh.qcols = (int)std::min<long long>(ld, round_up(cols, 8));
   sh.weight = (p >= Pb && p < Pb + nparam) || (p >= PbT && p < PbT + nparam);
   sh.transposed = p >= PbT && p < PbT + nparam;

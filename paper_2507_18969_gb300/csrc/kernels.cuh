@@ -223,7 +223,13 @@ cudaError_t launch_gemm_f32(const GemmF32& g, cudaStream_t st);
 
 // ---- BF16 path: fused operand production -----------------------------------------------------
 // The transposed copies YT[c][r] have a leading dimension ldT that is a multiple
-// of kRowsT (padding rows are written as zero), so that runs of rows are aligned.
+// of kRowsT, so that runs of rows are aligned. Entries at rows r >= b are
+// unspecified but finite: some producers write zeros up to the end of their tile,
+// others what their epilogue makes of an all-zero row (GELU of the biases'
+// product), or nothing. Consumers bound their contraction by b (the tensor maps
+// end there and read zeros beyond); only FP8's quantizer takes whole runs of
+// eight rows, into values that its maps then leave out, and into the scale, the
+// same in the encoder and the decoder.
 constexpr int kRowsT = 16;
 // LayerNorm forward writing xhat, rstd and the BF16 copies of X0 (row-major and transposed).
 // Grouped mode (rg != nullptr): row r uses g + rg[r] * gs and be + rg[r] * gs.

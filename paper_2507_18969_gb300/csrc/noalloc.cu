@@ -1,14 +1,12 @@
-// Range encoding without any device allocation.
+// Range encoding without any allocation per call, on the device or on the host.
 //
-// edpc_range_encode keeps a stream's coder state in registers from the first
-// symbol to the flush. This entry point codes through the session's kernels
-// instead (a prefix, coding and flush launch over coder states in memory), for
-// callers that may not allocate device memory: services that reserve their
-// whole device-memory budget at start-up and refuse later allocations, and
-// latency-sensitive loops that cannot absorb the device-wide synchronisation
-// cudaFree may perform. The states, output offsets and capacities are a fixed
-// array that is part of the library image itself: it exists on every GPU that
-// loads the library, from load until process exit.
+// edpc_range_encode makes no device allocation either (a stream's coder state
+// stays in registers from the first symbol to the flush), but holds the lengths
+// in a host buffer of its own. This entry point codes through the session's
+// kernels (a prefix, coding and flush launch over coder states in memory) and
+// reads back one overflow flag. The states, output offsets and capacities are a
+// fixed array that is part of the library image itself: it exists on every GPU
+// that loads the library, from load until process exit.
 #include <mutex>
 
 #include "kernels.cuh"
