@@ -527,10 +527,10 @@ int edpc_model_block_io(edpc_model* m, uint32_t block, float* s_in, float* s_out
  * are exact functions of the FP32 samples. *mi (host) receives
  * psi(k) + psi(N) - mean_i(psi(c_z(i) + 1) + psi(c_y(i) + 1)) in nats, FP64.
  * Runs on cuda_stream (NULL: the default stream) and waits for it.
- * The distances go through a device workspace of 8 N N' bytes (N' = N rounded
- * up to 64), at most 64 MiB, in panels of fewer rows where that or the free
- * memory does not hold them all (down to 64 rows, 512 N' bytes). It comes from
- * a memory pool of the library's own, one per device, which keeps up to 64 MiB
+ * But for small N, the distances go through a device workspace of 8 N N' bytes
+ * (N' = N rounded up to 64), at most 64 MiB, in panels of fewer rows where that
+ * or the free memory does not hold them all (down to 64 rows, 512 N' bytes). It
+ * comes from a memory pool of the library's own, one per device, which keeps up to 64 MiB
  * between calls for the life of the process; after a cudaDeviceReset of a
  * device this entry point must not be called on that device again.
  * Limits: 2 <= N <= 8192, 1 <= k <= min(64, N - 1), dz + dy <= 8192.

@@ -11,9 +11,10 @@
 // by the FP32 samples, whatever the order.
 // What bounds it is the FP32 pipe: a subtraction and a maximum per coordinate
 // and pair, halved by the symmetry and by packed subtractions (two per
-// instruction). With a CTA per sample that read every other sample from L2 and
-// selected over all N values with CTA-wide barriers, 2048 samples of 512 + 512
-// coordinates took 1525 us a call; now 205 (distances 139, selection 19).
+// instruction). With a CTA per sample that reads every other sample from L2 and
+// selects over all N values with CTA-wide barriers, 2048 samples of 512 + 512
+// coordinates took 1525 us a call; now 205 (distances 139, selection 19). That
+// form (ksg_row_kernel) remains for few samples, where it is the faster one.
 // The host then forms
 // psi(k) + psi(N) - mean(psi(c_z + 1) + psi(c_y + 1)) in FP64.
 #include <algorithm>
@@ -222,6 +223,96 @@ __global__ void ksg_select_kernel(const float* __restrict__ D, int R, int ld, in
   }
 }
 
+// Few samples: CTA i computes the distances of sample i to every sample j (a warp
+// per j, lanes over the coordinates, a butterfly maximum) into shared memory,
+// selects eps(i) with CTA-wide counts and counts c_z and c_y. One launch, no
+// workspace, a CTA per sample: the tiles above are too few CTAs by then, and each
+// runs through all the coordinates alone. The same exact differences and maxima,
+// so the same counts.
+constexpr int kRowThreads = 256;
+
+__device__ __forceinline__ int block_sum(int v, int* red) {
+  v = __reduce_add_sync(0xffffffffu, v);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (lane == 0) red[w] = v;
+  __syncthreads();
+  int s = 0;
+#pragma unroll
+  for (int q = 0; q < kRowThreads / 32; ++q) s += red[q];
+  return s;
+}
+
+__global__ void __launch_bounds__(kRowThreads) ksg_row_kernel(const float* __restrict__ Z, const float* __restrict__ Y,
+                                                              int N, int dz, int dy, int k, unsigned* __restrict__ cz,
+                                                              unsigned* __restrict__ cy) {
+  extern __shared__ __align__(16) float sm[];
+  float* zi = sm;        // dz
+  float* yi = zi + dz;   // dy
+  float* sdz = yi + dy;  // N
+  float* sdy = sdz + N;  // N
+  __shared__ int red[kRowThreads / 32];
+  const int i = blockIdx.x, t = threadIdx.x;
+  const int w = t >> 5, lane = t & 31;
+  for (int q = t; q < dz; q += kRowThreads) zi[q] = Z[(size_t)i * dz + q];
+  for (int q = t; q < dy; q += kRowThreads) yi[q] = Y[(size_t)i * dy + q];
+  __syncthreads();
+  for (int j = w; j < N; j += kRowThreads / 32) {
+    float a = 0.f, b = 0.f;
+    for (int q = lane; q < dz; q += 32) a = fmaxf(a, fabsf(Z[(size_t)j * dz + q] - zi[q]));
+    for (int q = lane; q < dy; q += 32) b = fmaxf(b, fabsf(Y[(size_t)j * dy + q] - yi[q]));
+    for (int o = 16; o > 0; o >>= 1) {
+      a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+      b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if (lane == 0) {
+      sdz[j] = a;
+      sdy[j] = b;
+    }
+  }
+  __syncthreads();
+  unsigned prefix = 0, mask = 0;
+  int kk = k;
+  for (int bit = 30; bit >= 0; --bit) {
+    int c = 0;
+    for (int j = t; j < N; j += kRowThreads) {
+      if (j == i) continue;
+      const unsigned u = __float_as_uint(fmaxf(sdz[j], sdy[j]));
+      c += ((u & mask) == prefix && ((u >> bit) & 1u) == 0u) ? 1 : 0;
+    }
+    c = block_sum(c, red);
+    if (c < kk) {
+      kk -= c;
+      prefix |= 1u << bit;
+    }
+    mask |= 1u << bit;
+  }
+  const float eps = __uint_as_float(prefix);
+  int nz = 0, ny = 0;
+  for (int j = t; j < N; j += kRowThreads) {
+    if (j == i) continue;
+    nz += sdz[j] < eps ? 1 : 0;
+    ny += sdy[j] < eps ? 1 : 0;
+  }
+  nz = block_sum(nz, red);
+  ny = block_sum(ny, red);
+  if (t == 0) {
+    cz[i] = (unsigned)nz;
+    cy[i] = (unsigned)ny;
+  }
+}
+
+// Which of the two: a tile's chain over max(dz, dy) coordinates against the row
+// kernel's N / 8 samples a warp. Calls in us, rows / tiles, dz = dy:
+//   32 samples: 39 / 41 (1 coordinate), 49 / 66 (512)     64: 42 / 41 (33), 42 / 44 (128), 49 / 66 (512)
+//   96: 50 / 43 (128), 50 / 52 (256), 62 / 65 (512)        128: 52 / 45 (128), 51 / 54 (256), 64 / 66 (512)
+//   160: 51 / 45 (128), 56 / 54 (256), 78 / 65 (512)
+// Rows that are not 16-byte aligned cost the row kernel more: 128: 76 / 68 (511).
+bool use_rows(int N, int dz, int dy, bool v16) {
+  return N < 64 || (N <= (v16 ? 128 : 96) && std::max(dz, dy) >= 2 * N);
+}
+static_assert(sizeof(float) * (8192 + 2 * 128) <= 48 * 1024, "the row kernel needs no attribute");
+
 // The distance workspace comes from a memory pool of the library's own, one per
 // device, that keeps at most kWorkspace bytes between calls (stream-ordered, so
 // concurrent calls on any threads and streams get buffers of their own; what
@@ -259,6 +350,57 @@ cudaError_t workspace_alloc(float** p, size_t bytes, cudaStream_t st) {
   return e != cudaSuccess ? e : cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, g_pool[dev], st);
 }
 
+// The tiled form: the distances into the workspace, then the counts.
+int launch_tiles(const float* Z, const float* Y, int N, int dz, int dy, int k, bool v16, uint32_t* cz, uint32_t* cy,
+                 cudaStream_t st) {
+  constexpr size_t kDistSmem = (size_t)kStages * 2 * kTile * kLd * sizeof(float);
+  constexpr size_t kListSmem = 128 * 1024;
+  static OncePerDevice once;
+  const cudaError_t attr = once_on_device(once, [] {
+    cudaError_t r =
+        cudaFuncSetAttribute(ksg_dist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(ksg_dist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(ksg_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem);
+    return r;
+  });
+  if (attr != cudaSuccess) return fail(EDPC_ECUDA, std::string("ksg attribute: ") + cudaGetErrorString(attr));
+  // The distances of all rows at once where they fit kWorkspace; else panels of rows.
+  const int ld = (int)round_up(N, kTile);
+  const size_t row = 2 * sizeof(float) * (size_t)ld;
+  int R = N;
+  if (row * N > kWorkspace) R = (int)(kWorkspace / row / kTile * kTile);
+  float* D = nullptr;
+  cudaError_t e = workspace_alloc(&D, row * R, st);
+  while (e == cudaErrorMemoryAllocation && R > kTile) {  // a smaller panel when memory is short
+    cudaGetLastError();
+    R = (int)round_up(R / 2, kTile);
+    e = workspace_alloc(&D, row * R, st);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(e == cudaErrorMemoryAllocation ? EDPC_ENOMEM : EDPC_ECUDA,
+                std::string("ksg workspace: ") + cudaGetErrorString(e));
+  }
+  const int warps = (int)std::min<size_t>(8, kListSmem / (sizeof(float) * ld));
+  const unsigned nt = ld / kTile;
+  for (int r0 = 0; r0 < N && e == cudaSuccess; r0 += R) {
+    const int rows = std::min(R, N - r0);
+    const unsigned tiles = rows == N ? nt * (nt + 1) / 2 : nt * div_up(rows, kTile);
+    auto k1 = v16 ? ksg_dist_kernel<true> : ksg_dist_kernel<false>;
+    e = launch_k(k1, dim3(tiles, 2), dim3(256), kDistSmem, st, Z, Y, N, dz, dy, D, ld, r0, rows);
+    if (e == cudaSuccess)
+      e = launch_k(ksg_select_kernel, dim3(div_up(rows, warps)), dim3(32 * warps), sizeof(float) * ld * warps, st,
+                   (const float*)D, rows, ld, k, (unsigned*)cz + r0, (unsigned*)cy + r0);
+  }
+  {
+    const cudaError_t f = cudaFreeAsync(D, st);
+    if (e == cudaSuccess) e = f;
+  }
+  return e == cudaSuccess ? EDPC_OK : fail(EDPC_ECUDA, std::string("ksg: ") + cudaGetErrorString(e));
+}
+
 // psi(x) for x >= 1: recurrence up to x >= 10, then the asymptotic series
 // ln x - 1/(2x) - sum_n B_2n / (2n x^2n) (Abramowitz & Stegun 6.3.6, 6.3.18).
 double digamma_ge1(double x) {
@@ -285,55 +427,16 @@ extern "C" int edpc_ksg_mi(const float* Z, const float* Y, uint32_t N, uint32_t 
   if (N < 2 || N > 8192) return fail(EDPC_EINVAL, "N must be in [2, 8192]");
   if (k < 1 || k >= N || k > 64) return fail(EDPC_EINVAL, "k must be in [1, min(64, N - 1)]");
   if (dz < 1 || dy < 1 || dz + dy > 8192) return fail(EDPC_EINVAL, "dz, dy >= 1 and dz + dy <= 8192");
-  constexpr size_t kDistSmem = (size_t)kStages * 2 * kTile * kLd * sizeof(float);
-  constexpr size_t kListSmem = 128 * 1024;
-  static OncePerDevice once;
-  const cudaError_t attr = once_on_device(once, [] {
-    cudaError_t r =
-        cudaFuncSetAttribute(ksg_dist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
-    if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(ksg_dist_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDistSmem);
-    if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(ksg_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem);
-    return r;
-  });
-  if (attr != cudaSuccess) return fail(EDPC_ECUDA, std::string("ksg attribute: ") + cudaGetErrorString(attr));
-  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  NoPdl scope;
-  // The distances of all rows at once where they fit kWorkspace; else panels of rows.
-  const int ld = (int)round_up(N, kTile);
-  const size_t row = 2 * sizeof(float) * (size_t)ld;
-  int R = (int)N;
-  if (row * N > kWorkspace) R = (int)(kWorkspace / row / kTile * kTile);
-  float* D = nullptr;
-  cudaError_t e = workspace_alloc(&D, row * R, st);
-  while (e == cudaErrorMemoryAllocation && R > kTile) {  // a smaller panel when memory is short
-    cudaGetLastError();
-    R = (int)round_up(R / 2, kTile);
-    e = workspace_alloc(&D, row * R, st);
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(e == cudaErrorMemoryAllocation ? EDPC_ENOMEM : EDPC_ECUDA,
-                std::string("ksg workspace: ") + cudaGetErrorString(e));
-  }
   const bool v16 = dz % 4 == 0 && dy % 4 == 0 &&
                    ((reinterpret_cast<uintptr_t>(Z) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
-  const int warps = (int)std::min<size_t>(8, kListSmem / (sizeof(float) * ld));
-  const unsigned nt = ld / kTile;
-  for (int r0 = 0; r0 < (int)N && e == cudaSuccess; r0 += R) {
-    const int rows = std::min(R, (int)N - r0);
-    const unsigned tiles = rows == (int)N ? nt * (nt + 1) / 2 : nt * div_up(rows, kTile);
-    auto k1 = v16 ? ksg_dist_kernel<true> : ksg_dist_kernel<false>;
-    e = launch_k(k1, dim3(tiles, 2), dim3(256), kDistSmem, st, Z, Y, (int)N, (int)dz, (int)dy, D, ld, r0, rows);
-    if (e == cudaSuccess)
-      e = launch_k(ksg_select_kernel, dim3(div_up(rows, warps)), dim3(32 * warps), sizeof(float) * ld * warps, st,
-                   (const float*)D, rows, ld, (int)k, (unsigned*)cz + r0, (unsigned*)cy + r0);
-  }
-  {
-    const cudaError_t f = cudaFreeAsync(D, st);
-    if (e == cudaSuccess) e = f;
-  }
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  NoPdl scope;
+  cudaError_t e = cudaSuccess;
+  if (use_rows((int)N, (int)dz, (int)dy, v16))
+    e = launch_k(ksg_row_kernel, dim3(N), dim3(kRowThreads), sizeof(float) * ((size_t)dz + dy + 2 * (size_t)N), st, Z, Y,
+                 (int)N, (int)dz, (int)dy, (int)k, (unsigned*)cz, (unsigned*)cy);
+  else
+    EDPC_TRY(launch_tiles(Z, Y, (int)N, (int)dz, (int)dy, (int)k, v16, cz, cy, st));
   std::vector<uint32_t> hz(N), hy(N);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hz.data(), cz, 4 * (size_t)N, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hy.data(), cy, 4 * (size_t)N, cudaMemcpyDeviceToHost, st);
