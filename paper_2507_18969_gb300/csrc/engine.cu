@@ -749,7 +749,6 @@ int Model::fdm_bwd_call(const StepIO& io, cudaStream_t st) {
 }
 
 int Model::backward_f32(const StepIO& io, cudaStream_t st) {
-  nfork_ = 0;
   auto one = [&](const float* X, int cols, size_t off) {
     ColsumJobs cj{};
     cj.job[0] = {X, nullptr, d.b, cols, cols, G + off};
@@ -1331,8 +1330,7 @@ int Model::colsums(ColsumJobs cj, cudaStream_t st) {
 
 // `to` waits for everything launched so far on `from`.
 int Model::fork_to(cudaStream_t from, cudaStream_t to) {
-  if (nfork_ >= kForks) return fail(EDPC_EINVAL, "too many side-stream forks in one step");
-  cudaEvent_t e = fork[nfork_++];
+  cudaEvent_t e = fork[nfork_++ % kForks];
   EDPC_CUDA(cudaEventRecord(e, from));
   EDPC_CUDA(cudaStreamWaitEvent(to, e, 0));
   return EDPC_OK;
@@ -1404,7 +1402,6 @@ EmbAdam Model::emb_adam(const StepIO& io) const {
 }
 
 int Model::forward_bf16(const StepIO& io, cudaStream_t st) {
-  nfork_ = 0;  // the waits on the previous pass's forks have all been issued; a forward pass may be repeated alone
   const bool f8m = precision == EDPC_FP8E4M3;
   if (f8m) {
     std::fill(f8_done.begin(), f8_done.end(), 0);
@@ -1468,7 +1465,6 @@ int Model::fdm_bwd_joined(const StepIO& io, cudaStream_t st) {
 
 int Model::backward_bf16(const StepIO& io, cudaStream_t st) {
   const int kH = d.k * d.H;
-  nfork_ = 0;  // (so has the wait on the forward pass's fork)
   const bool f8m = precision == EDPC_FP8E4M3;
   // the dX GEMMs read FP8's transposed shadows (delayed update: made during the previous step)
   if (f8m && !delayed) EDPC_CUDA(cudaStreamWaitEvent(st, tr_ev, 0));

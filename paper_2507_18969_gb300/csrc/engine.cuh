@@ -78,7 +78,9 @@ class Model {
   TcPlan tcp;
   cudaStream_t side = nullptr;                             // dW GEMMs
   cudaStream_t side2 = nullptr;                            // column sums, and Adam layer by layer
-  static constexpr int kForks = 5 * kMaxBlocks + 16;
+  // Fork and join events, used in turn: a wait stands for the record it was
+  // issued after, so an event may be recorded again as soon as its wait is issued.
+  static constexpr int kForks = 16;
   cudaEvent_t fork[kForks] = {};
   cudaEvent_t tr_ev = nullptr;                             // transposed weight copies ready
   // FDM update off the critical path (BF16/FP8): dx' on the step's stream, the
@@ -212,7 +214,7 @@ class Model {
  private:
   void* arena_ = nullptr;
   size_t arena_bytes_ = 0;
-  int nfork_ = 0;
+  unsigned nfork_ = 0;
   bool tuning_ = false;  // the tuner times the kernels that the tile codes name
   Advance advance_of(const StepIO& io) const;
   EmbAdam emb_adam(const StepIO& io) const;
