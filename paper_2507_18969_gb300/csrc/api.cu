@@ -436,7 +436,7 @@ struct edpc_session {
   // An event-record node between two kernels costs the programmatic edge
   // between them: around the two FDM launches such nodes left gaps of 5, 15
   // and 12 us in the 425 us step of the 64 MiB mix. So the timed graphs
-  // (x_chunk: `chunk` steps, instantiated twice with separate events and
+  // (x_timed: timed_steps steps, instantiated twice with separate events and
   // launched alternately; x_one_t: one step) are made when profiling is first
   // turned on.
   // run_steps and run_min: capturing, instantiating and destroying a graph takes
@@ -450,15 +450,19 @@ struct edpc_session {
   // They meet at 500 steps (small models) to 1700 (64 MiB mix, 64 streams).
   // Schedules that keep an FDM update running under the next step's layers join
   // it at a graph's end, so they have `chunk` steps a graph, from as many steps on.
-  cudaGraph_t g_run = nullptr, g_one = nullptr, g_chunk = nullptr, g_one_t = nullptr;
-  cudaGraphExec_t x_run = nullptr, x_one = nullptr, x_chunk[2] = {}, x_one_t = nullptr;
+  // timed_steps: two graphs of 16 steps keep the GPU busy while the host reads the
+  // events of the one before. With 64 a profiled session of 200 steps of a 16-block
+  // model took 188 ms, 112 of them to make and destroy these graphs; now 86 and 22.
+  cudaGraph_t g_run = nullptr, g_one = nullptr, g_timed = nullptr, g_one_t = nullptr;
+  cudaGraphExec_t x_run = nullptr, x_one = nullptr, x_timed[2] = {}, x_one_t = nullptr;
   static constexpr int kRunSteps = 8, kRunMin = 1024;
   int run_steps = kRunSteps;
+  int timed_steps = 16;
   int graph_kernels = 0;  // kernels per step
 
-  // FDM kernel timing: event set k of chunk execution p is tev[p * chunk + k];
-  // the one-step graph (and eager steps) use the sets after those. Made when
-  // profiling is first turned on.
+  // FDM kernel timing: event set k of the timed graph's execution p is
+  // tev[p * timed_steps + k] (eager steps use these in turn); the one-step graph
+  // uses the set after those. Made when profiling is first turned on.
   bool profiling = false;
   static constexpr int kChunk = 64;
   static constexpr int kEvSets = 2 * kChunk + 1;
@@ -486,11 +490,11 @@ struct edpc_session {
 edpc_session::~edpc_session() {
   if (st) cudaStreamSynchronize(st);
   if (st_coder) cudaStreamSynchronize(st_coder);
-  for (auto& x : x_chunk)
+  for (auto& x : x_timed)
     if (x) cudaGraphExecDestroy(x);
   for (auto& x : {x_one, x_run, x_one_t})
     if (x) cudaGraphExecDestroy(x);
-  for (auto& g : {g_chunk, g_one, g_run, g_one_t})
+  for (auto& g : {g_timed, g_one, g_run, g_one_t})
     if (g) cudaGraphDestroy(g);
   for (auto& e : ev_model)
     if (e) cudaEventDestroy(e);
@@ -611,7 +615,7 @@ int edpc_session::capture(int nsteps, int set0, cudaGraph_t* g) {
 int edpc_session::capture_graph() {
   has_adam_ev = model.side_fdm != nullptr;
   if (!use_graph || steps_total == 0) return EDPC_OK;
-  run_steps = model.side_fdm ? kChunk : kRunSteps;
+  if (model.side_fdm) run_steps = timed_steps = kChunk;
   EDPC_TRY(capture(1, -1, &g_one));
   EDPC_CUDA(cudaGraphInstantiate(&x_one, g_one, 0));
   size_t nn = 0;
@@ -632,31 +636,32 @@ int edpc_session::capture_graph() {
 
 // The events and the graphs that profiling uses.
 int edpc_session::capture_timed() {
-  for (auto& set : tev)
-    for (auto& e : set)
+  for (int k = 0; k <= 2 * timed_steps; ++k)
+    for (auto& e : tev[k])
       if (!e) EDPC_CUDA(cudaEventCreate(&e));
   if (!use_graph || steps_total == 0 || x_one_t) return EDPC_OK;
   EDPC_CUDA(cudaStreamSynchronize(st));
   EDPC_TRY(model.flush(st));  // an eager step's FDM update is waited for outside the capture
-  if (!g_one_t) EDPC_TRY(capture(1, 2 * kChunk, &g_one_t));
-  if (steps_total >= (uint64_t)kChunk) {
-    if (!g_chunk) EDPC_TRY(capture(kChunk, 0, &g_chunk));
-    for (auto& x : x_chunk)
-      if (!x) EDPC_CUDA(cudaGraphInstantiate(&x, g_chunk, 0));
-    // the second instantiation records into event sets kChunk .. 2 kChunk - 1
+  if (!g_one_t) EDPC_TRY(capture(1, 2 * timed_steps, &g_one_t));
+  if (steps_total >= (uint64_t)timed_steps) {
+    if (!g_timed) EDPC_TRY(capture(timed_steps, 0, &g_timed));
+    for (auto& x : x_timed)
+      if (!x) EDPC_CUDA(cudaGraphInstantiate(&x, g_timed, 0));
+    // the second instantiation records into event sets timed_steps .. 2 timed_steps - 1
     size_t nn = 0;
-    EDPC_CUDA(cudaGraphGetNodes(g_chunk, nullptr, &nn));
+    EDPC_CUDA(cudaGraphGetNodes(g_timed, nullptr, &nn));
     std::vector<cudaGraphNode_t> nodes(nn);
-    EDPC_CUDA(cudaGraphGetNodes(g_chunk, nodes.data(), &nn));
+    EDPC_CUDA(cudaGraphGetNodes(g_timed, nodes.data(), &nn));
     for (auto nd : nodes) {
       cudaGraphNodeType t;
       EDPC_CUDA(cudaGraphNodeGetType(nd, &t));
       if (t != cudaGraphNodeTypeEventRecord) continue;
       cudaEvent_t e;
       EDPC_CUDA(cudaGraphEventRecordNodeGetEvent(nd, &e));
-      for (int k = 0; k < kChunk; ++k)
+      for (int k = 0; k < timed_steps; ++k)
         for (int q = 0; q < kEv; ++q)
-          if (e == tev[k][q]) EDPC_CUDA(cudaGraphExecEventRecordNodeSetEvent(x_chunk[1], nd, tev[kChunk + k][q]));
+          if (e == tev[k][q])
+            EDPC_CUDA(cudaGraphExecEventRecordNodeSetEvent(x_timed[1], nd, tev[timed_steps + k][q]));
     }
   }
   EDPC_CUDA(cudaGraphInstantiate(&x_one_t, g_one_t, 0));
@@ -693,24 +698,24 @@ int edpc_session::launch_steps(uint64_t n) {
     if (encoder && pipeline && j % chunk == 0 && j >= (uint64_t)(2 * chunk))
       EDPC_CUDA(cudaStreamWaitEvent(st, ev_coder[(j / chunk) % 2], 0));
     uint64_t adv = 1;
-    if (profiling && x_chunk[0] && fits(j, chunk)) {
-      const int p = (int)((j / chunk) % 2);
-      for (int q = 0; q < chunk; ++q) EDPC_TRY(harvest(p * chunk + q));
+    if (profiling && x_timed[0] && fits(j, timed_steps)) {
+      const int p = (int)((j / timed_steps) % 2);
+      for (int q = 0; q < timed_steps; ++q) EDPC_TRY(harvest(p * timed_steps + q));
       EDPC_TRY(model.flush(st));  // an eager step's FDM update may still run on its own stream
-      EDPC_CUDA(cudaGraphLaunch(x_chunk[p], st));
-      for (int q = 0; q < chunk; ++q) tev_live[p * chunk + q] = true;
-      adv = (uint64_t)chunk;
+      EDPC_CUDA(cudaGraphLaunch(x_timed[p], st));
+      for (int q = 0; q < timed_steps; ++q) tev_live[p * timed_steps + q] = true;
+      adv = (uint64_t)timed_steps;
     } else if (!profiling && x_run && fits(j, run_steps)) {
       EDPC_TRY(model.flush(st));
       EDPC_CUDA(cudaGraphLaunch(x_run, st));
       adv = (uint64_t)run_steps;
     } else if (x_one && !model.delayed) {  // (the delayed update alternates parities: eager)
-      const int set = 2 * kChunk;
+      const int set = 2 * timed_steps;
       if (profiling) EDPC_TRY(harvest(set));
       EDPC_CUDA(cudaGraphLaunch(profiling ? x_one_t : x_one, st));
       if (profiling) tev_live[set] = true;
     } else {
-      const int set = (int)(j % (2 * kChunk));
+      const int set = (int)(j % (2 * timed_steps));
       if (profiling) {
         EDPC_TRY(harvest(set));
         for (int q = 0; q < kEv; ++q) model.ev_fdm[q] = tev[set][q];
