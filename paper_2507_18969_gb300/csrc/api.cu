@@ -439,14 +439,17 @@ struct edpc_session {
   // (x_timed: timed_steps steps, instantiated twice with separate events and
   // launched alternately; x_one_t: one step) are made when profiling is first
   // turned on.
-  // run_steps and run_min: capturing, instantiating and destroying a graph takes
-  // time in proportion to its nodes (about 60 a step), and all that the longer
-  // graph saves is 1 to 2.5 us a step of hand-over between launches. So x_run
-  // is made for sessions of run_min steps and more only. Whole compressions, one-step
-  // graph alone / with the 8-step graph / with a 16-step one, in ms:
-  //   default model, FP32, 4 streams     24 steps 2.3 / 3.5 / 4.8     512: 36.2 / 36.0 / 37.1   2048: 142.0 / 137.2 / 138.9
-  //   64 MiB mix's model, 512 streams    24 steps 8.7 / 10.5 / 12.7  1024: 313.8 / 314.4 / 316.9  2048: 628.5 / 625.9 / 628.4
-  //   1 GiB mix's model, 16 streams      24 steps 8.8 / 11.3 / 13.9  1024: 307.6 / 307.4 / 310.8  2048: 611.9 / 609.9 / 613.1
+  // run_steps: capturing, instantiating and destroying a graph takes time in
+  // proportion to its nodes (about 60 a step), and all that a longer graph saves
+  // is 1 to 2.5 us a step of hand-over between launches. So x_run has eight steps
+  // and is made from kRunMin steps on. Whole compressions in ms, with the one-step
+  // graph alone / with 8 steps / with 16 steps a graph:
+  //   default model, FP32, 4 streams    24 steps: 2.3 / 3.5 / 4.8        512: 36.2 / 36.0 / 37.1
+  //                                     2048 steps: 142.0 / 137.2 / 138.9
+  //   64 MiB mix's model, 512 streams   24 steps: 8.7 / 10.5 / 12.7      1024: 313.8 / 314.4 / 316.9
+  //                                     2048 steps: 628.5 / 625.9 / 628.4
+  //   1 GiB mix's model, 16 streams     24 steps: 8.8 / 11.3 / 13.9      1024: 307.6 / 307.4 / 310.8
+  //                                     2048 steps: 611.9 / 609.9 / 613.1
   // They meet at 500 steps (small models) to 1700 (64 MiB mix, 64 streams).
   // Schedules that keep an FDM update running under the next step's layers join
   // it at a graph's end, so they have `chunk` steps a graph, from as many steps on.
